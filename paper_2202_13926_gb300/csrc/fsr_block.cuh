@@ -1006,24 +1006,31 @@ __device__ __forceinline__ void iterate(double (&zr)[S], double (&zi)[S], double
     }
 }
 
+// w of Eq. (5) on a known pixel, and w_f of Eq. (9).
+template <typename T>
+__device__ __forceinline__ T w0_value(const MethodArgs& mth, int m, int n) {
+    const T dm = T(m) - T(S - 1) / T(2), dn = T(n) - T(S - 1) / T(2);
+    return pow(T(mth.rho), sqrt(dm * dm + dn * dn));
+}
+template <typename T>
+__device__ __forceinline__ T wf_value(const MethodArgs& mth, int k, int l) {
+    if (!mth.freq_weight) return T(1);
+    const T half = T(S) / T(2);
+    const T kt = half - fabs(T(k) - half), lt = half - fabs(T(l) - half);
+    const T r = sqrt(kt * kt / T(S * S) + lt * lt / T(S * S));
+    const T b = T(1) - sqrt(T(2)) * r;
+    return b * b;
+}
+
 // Shared-memory tables of one CTA: Eqs. (5) and (9) and cos/sin(2 pi t / S).
 template <typename T>
 __device__ __forceinline__ void cta_tables(const MethodArgs& mth, T* sw0, T* swf,
                                            typename Vec2<T>::type* scs) {
     using T2 = typename Vec2<T>::type;
-    const T half = T(S) / T(2);
     for (int i = threadIdx.x; i < S * S; i += blockDim.x) {
         const int m = i / S, n = i % S;
-        const T dm = T(m) - T(S - 1) / T(2), dn = T(n) - T(S - 1) / T(2);
-        sw0[i] = pow(T(mth.rho), sqrt(dm * dm + dn * dn));
-        T wfv = T(1);
-        if (mth.freq_weight) {
-            const T kt = half - fabs(T(m) - half), lt = half - fabs(T(n) - half);
-            const T r = sqrt(kt * kt / T(S * S) + lt * lt / T(S * S));
-            const T b = T(1) - sqrt(T(2)) * r;
-            wfv = b * b;
-        }
-        swf[m * WFS + n] = wfv;
+        sw0[i] = w0_value<T>(mth, m, n);
+        swf[m * WFS + n] = wf_value<T>(mth, m, n);
     }
     for (int t = threadIdx.x; t < S; t += blockDim.x) {
         T2 v;

@@ -212,14 +212,30 @@ int read_status(fsr_handle* h) {
                 st);
 }
 
-// FP32 single image (and any image of a support smaller than 32): a
-// one-image work table in one of the handle's table slots (used in turn; a
+// FP32 single image (and any image of a support smaller than 32).  Few blocks
+// of S = 32: the CTA-per-block kernel with the image in its parameters.  Else
+// a one-image work table in one of the handle's table slots (used in turn; a
 // slot is reused once the launch that read it has finished), then the batch
 // kernel with the handle's schedule.
 int enqueue_single_fp32(fsr_handle* h, const float* img, const uint8_t* mask, int height, int width, int pitch,
                         const fsr_params* p, float* out, cudaStream_t stream) {
-    const int slot = (int)(h->single_next++ % fsr_handle::kSingleSlots);
     cudaError_t e;
+    const fsrk::Schedule sc = h->sched[p->precision == FSR_FP64_DEBUG ? 1 : 0][b_index(p->block)];
+    const long long blocks = fsr_num_blocks(height, width, p->block);
+    if (p->precision == FSR_FP32 && p->block + 2 * p->border == fsrk::S && p->update == FSR_UPDATE_SINGLE &&
+        sc.warps == fsrk::kWarpsFp32 && !h->inject_tile_fault &&
+        blocks <= (long long)fsrk::kCoopBlocksPerSm * h->sm_count) {
+        // few blocks: the arguments travel with the launch, no table
+        fsrk::BatchArgs a = {};
+        a.total = blocks;
+        a.mth = method_args(p);
+        a.empty = h->d_empty;
+        const fsrk::ImageArgs im = image_args(img, mask, out, p->seq_out, height, width, pitch, p->iters, p->block);
+        if ((e = fsrk::launch_coop(a, p->block, &im, stream)) != cudaSuccess)
+            return fail(h, FSR_ERR_CUDA, "kernel launch failed: %s", cudaGetErrorString(e));
+        return ok(h);
+    }
+    const int slot = (int)(h->single_next++ % fsr_handle::kSingleSlots);
     if (h->single_used[slot] && (e = cudaEventSynchronize(h->single_ev[slot])) != cudaSuccess)
         return fail(h, FSR_ERR_CUDA, "waiting for a table slot: %s", cudaGetErrorString(e));
     char* host = static_cast<char*>(h->h_single) + (size_t)slot * fsr_handle::kSingleSlotBytes;
@@ -237,7 +253,6 @@ int enqueue_single_fp32(fsr_handle* h, const float* img, const uint8_t* mask, in
     if (total < 0) return FSR_ERR_CUDA;
     if ((e = cudaMemcpyAsync(dev, host, table_bytes(1), cudaMemcpyHostToDevice, stream)) != cudaSuccess)
         return fail(h, FSR_ERR_CUDA, "table upload: %s", cudaGetErrorString(e));
-    const fsrk::Schedule sc = h->sched[p->precision == FSR_FP64_DEBUG ? 1 : 0][b_index(p->block)];
     fsrk::BatchArgs a = batch_args(h, dev, 1, total, p, sc.chunk);
     a.empty = h->d_empty;
     a.tx_extra = h->inject_tile_fault ? 16 : 0;

@@ -1,0 +1,76 @@
+// Instantiations and launches of the CTA-per-block FP32 kernels (fsr_coop.cuh).
+#include "fsr_coop.cuh"
+
+namespace fsrk {
+namespace {
+
+template <int B>
+cudaError_t configure_b() {
+    cudaError_t e;
+    const int bytes = (int)sizeof(coop::Smem);
+    const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    if ((e = cudaFuncSetAttribute(coop::fsr_coop_kernel<B, true>, at, bytes)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(coop::fsr_coop_kernel<B, false>, at, bytes)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(coop::fsr_coop_reuse_kernel<B, 1>, at, bytes)) != cudaSuccess) return e;
+    return cudaFuncSetAttribute(coop::fsr_coop_reuse_kernel<B, kReuseSegs>, at, bytes);
+}
+
+template <int B>
+cudaError_t launch_b(const BatchArgs& a, const ImageArgs* one, cudaStream_t stream) {
+    const size_t smem = sizeof(coop::Smem);
+    if (one) coop::fsr_coop_kernel<B, true><<<(unsigned)a.total, coop::T, smem, stream>>>(a, *one);
+    else coop::fsr_coop_kernel<B, false><<<(unsigned)a.total, coop::T, smem, stream>>>(a, ImageArgs());
+    return cudaGetLastError();
+}
+
+template <int B, int NSEG>
+cudaError_t launch_reuse_n(const ReuseLaunchN<NSEG>& a, cudaStream_t stream) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)a.total);
+    cfg.blockDim = dim3(coop::T);
+    cfg.dynamicSmemBytes = sizeof(coop::Smem);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, coop::fsr_coop_reuse_kernel<B, NSEG>, a);
+}
+
+template <int B>
+cudaError_t launch_reuse_b(const ReuseLaunch& a, cudaStream_t stream) {
+    return a.nseg == 1 ? launch_reuse_n<B, 1>(one_image(a), stream) : launch_reuse_n<B, kReuseSegs>(a, stream);
+}
+
+}  // namespace
+
+cudaError_t configure_coop() {
+    cudaError_t e;
+    if ((e = configure_b<2>()) != cudaSuccess) return e;
+    if ((e = configure_b<4>()) != cudaSuccess) return e;
+    if ((e = configure_b<8>()) != cudaSuccess) return e;
+    return configure_b<16>();
+}
+
+cudaError_t launch_coop(const BatchArgs& a, int B, const ImageArgs* one, cudaStream_t stream) {
+    switch (B) {
+        case 2: return launch_b<2>(a, one, stream);
+        case 4: return launch_b<4>(a, one, stream);
+        case 8: return launch_b<8>(a, one, stream);
+        case 16: return launch_b<16>(a, one, stream);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+cudaError_t launch_coop_reuse(const ReuseLaunch& a, int B, cudaStream_t stream) {
+    switch (B) {
+        case 2: return launch_reuse_b<2>(a, stream);
+        case 4: return launch_reuse_b<4>(a, stream);
+        case 8: return launch_reuse_b<8>(a, stream);
+        case 16: return launch_reuse_b<16>(a, stream);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+}  // namespace fsrk

@@ -1,0 +1,457 @@
+// FP32 FSR at S = 32 with a CTA of four warps on one support block, for calls
+// with few blocks in flight: the 32 x 32 spectrum is spread over 128 threads,
+// 8 components each.
+//
+// What bounds it: the K iterations of a block are a serial chain (the argmax
+// of Eq. (8) needs the residual of Eq. (12), which needs the last argmax), so
+// such a call pays the latency of one iteration K times.  One warp per block
+// (fsr_block.cuh) walks 32 components per lane in every iteration; here the
+// update and the objective of a thread are 8 independent components, and one
+// CTA barrier per iteration joins the four warps' maxima.
+//
+// The arithmetic of every component, of both transforms, of the objective and
+// of the target pixels is that of fsr_block.cuh operation by operation, and
+// so is the selection rule: the results are the same bit for bit.
+//
+// Spectrum layout: warp w holds rows 8w .. 8w + 7, lane (r, g) of it the
+// columns g, g + 4, ..., g + 28 of row 8w + r (r = lane / 4, g = lane % 4).
+// A half-warp then reads 4 rows of 4 consecutive W entries; the row stride of
+// 68 entries of 8 bytes puts them on distinct banks for every shift (u, v).
+// W is stored twice in both directions (64 rows of 64 entries), so the shifted
+// entry W[k-u][l-v] of a thread is one subtraction away from a fixed address:
+// no wrap of either index on the chain from the pick to the W loads.
+//
+// Measured (alone on an SM, cycles at 1.98 GHz): one iteration 1,130 with one
+// warp per block, 457 here; of it about 40 the W load, 60 the update,
+// objective and maximum, 70 two warp reductions, 90 the barrier and the
+// candidates through shared memory.  What a thread may publish, and the
+// target pixels of the previous pick, are computed while the reductions run.
+// 8 and 16 warps per block: 480-600 (more candidates to read and more warps
+// at the barrier), at more issue slots.
+//
+// Transforms: the radix-2 decimation-in-time FFT of length 32 splits over the
+// warps.  Warp q takes the inputs of rows (columns) = brev2(q) mod 4, does
+// the three stages inside its 8 points in registers, and after one exchange
+// through shared memory the last two stages of the points t, t + 8, t + 16,
+// t + 24 for t = 2q, 2q + 1.  A thread so runs about 200 instructions per
+// transform where a lane of the one-warp kernel runs 1,200 of straight code,
+// most of whose time a block that runs alone spends fetching instructions.
+#pragma once
+
+#include "fsr_launch.h"
+
+namespace fsrk {
+namespace coop {
+
+constexpr int NW = 4;                    // warps per block
+constexpr int T = 32 * NW;               // threads per block
+constexpr int G = 4;                     // lanes per row
+constexpr int NC = S / G;                // components per thread
+constexpr int RPW = S / NW;              // rows per warp
+constexpr int WS = 68;                   // W row stride (float2)
+constexpr int AS = S + 1;                // row stride of the transform buffers (float2)
+constexpr int H1 = S / 2 + 1;            // w_f quadrant: indices 0 .. S/2
+
+struct Smem {
+    float2 A[S * AS];                    // support (f, w), first transform, spectrum Z
+    float2 W[2 * S * WS];                // exchange buffer of the transforms, then the W rows
+    float4 slot[2][NW];                  // candidates of the warps: maximum, shift offset, coefficient
+    float w0[S / 2 * S / 2];             // Eq. (5), one quadrant (symmetric)
+    float wf[H1 * H1];                   // Eq. (9), one quadrant (symmetric)
+    float2 cs[S];                        // cos, sin of 2 pi t / S
+    unsigned flags[NW];                  // per warp: 1 = a pixel of the support is available, 2 = an unknown target pixel
+    unsigned dmax[NW];
+};
+
+__device__ __forceinline__ int fold(int m) { return m < S / 2 ? m : S - 1 - m; }   // w0: m and S-1-m are alike
+__device__ __forceinline__ int foldf(int k) { return k <= S / 2 ? k : S - k; }      // w_f: k and S-k are alike
+
+// The tables of the CTA: pairs (m, n) with m <= n, both ways round.  Not
+// unrolled: a CTA that runs one block fetches this code cold, and the fetch,
+// not the arithmetic, is its time.
+__device__ __forceinline__ void tables(const MethodArgs& mth, Smem* sm) {
+#pragma unroll 1
+    for (int i = threadIdx.x; i < H1 * (H1 + 1) / 2; i += T) {
+        // rows r and 16 - r of the triangle side by side: 18 entries
+        const int r = i / (H1 + 1), c = i % (H1 + 1);
+        const bool first = c < H1 - r;
+        const int m = first ? r : H1 - 1 - r, n = first ? r + c : c - 1;
+        sm->wf[m * H1 + n] = sm->wf[n * H1 + m] = wf_value<float>(mth, m, n);
+        if (n < S / 2) sm->w0[m * (S / 2) + n] = sm->w0[n * (S / 2) + m] = w0_value<float>(mth, m, n);
+    }
+    if (threadIdx.x < S) sm->cs[threadIdx.x] = make_float2(float(cos_2pi32(threadIdx.x)), float(sin_2pi32(threadIdx.x)));
+}
+
+// One butterfly of the FFT, twiddle e^{-j 2 pi tw / 32} = c + j s, with the
+// products rounded as in fft32: of each of x_r = b_r c - b_i s and x_i = b_r s
+// + b_i c one product is rounded and the other fused.  fft32's choice is the
+// compiler's: b_r c and b_i c are the fused ones, but for tw = 4 b_r s in x_i
+// and for tw = 12 b_i s in x_r (found by comparing all choices bit for bit).
+// c = 1, s = -0 and c = 0, s = -1 give fft32's multiplication-free cases.
+__device__ __forceinline__ void butterfly(float2& a, float2& b, float c, float s, int tw) {
+    const bool t4 = tw == 4, t12 = tw == 12;
+    const float xr = __fmaf_rn(t12 ? -b.y : b.x, t12 ? s : c, t12 ? __fmul_rn(b.x, c) : -__fmul_rn(b.y, s));
+    const float xi = __fmaf_rn(t4 ? b.x : b.y, t4 ? s : c, t4 ? __fmul_rn(b.y, c) : __fmul_rn(b.x, s));
+    b.x = __fsub_rn(a.x, xr);
+    b.y = __fsub_rn(a.y, xi);
+    a.x = __fadd_rn(a.x, xr);
+    a.y = __fadd_rn(a.y, xi);
+}
+__device__ __forceinline__ void butterfly_one(float2& a, float2& b) {   // twiddle 1
+    const float2 x = b;
+    b = make_float2(__fsub_rn(a.x, x.x), __fsub_rn(a.y, x.y));
+    a = make_float2(__fadd_rn(a.x, x.x), __fadd_rn(a.y, x.y));
+}
+__device__ __forceinline__ void butterfly_mj(float2& a, float2& b) {    // twiddle -j
+    const float2 x = make_float2(b.y, -b.x);
+    b = make_float2(__fsub_rn(a.x, x.x), __fsub_rn(a.y, x.y));
+    a = make_float2(__fadd_rn(a.x, x.x), __fadd_rn(a.y, x.y));
+}
+
+// index of point i (bit-reversed position 8q + i) of warp q's 8 inputs
+__device__ __forceinline__ constexpr int in_index(int q2, int i) { return 4 * (((i & 1) << 2) | (i & 2) | (i >> 2)) + q2; }
+
+// stages 1-3 on the 8 points of a thread, exchange through X, stages 4-5.
+// e[2 h + ..]: on return e[tt][p] is output t + 8 p, t = 2 q + tt.
+__device__ __forceinline__ void fft32_split(float2 (&x)[8], float2 (&e)[2][4], float2* X, const float2* cs, int q,
+                                            int lane) {
+#pragma unroll
+    for (int i = 0; i < 8; i += 2) butterfly_one(x[i], x[i + 1]);
+#pragma unroll
+    for (int i = 0; i < 8; i += 4) {
+        butterfly_one(x[i], x[i + 2]);
+        butterfly_mj(x[i + 1], x[i + 3]);
+    }
+    butterfly_one(x[0], x[4]);
+    butterfly(x[1], x[5], float(cos_2pi32(4)), float(-sin_2pi32(4)), 4);
+    butterfly_mj(x[2], x[6]);
+    butterfly(x[3], x[7], float(cos_2pi32(12)), float(-sin_2pi32(12)), 12);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) X[(8 * q + i) * AS + lane] = x[i];
+    __syncthreads();
+#pragma unroll
+    for (int tt = 0; tt < 2; ++tt) {
+        const int t = 2 * q + tt;
+#pragma unroll
+        for (int p = 0; p < 4; ++p) e[tt][p] = X[(t + 8 * p) * AS + lane];
+        const float2 c2 = cs[2 * t], c1 = cs[t], c9 = cs[t + 8];
+        butterfly(e[tt][0], e[tt][1], c2.x, -c2.y, 2 * t);
+        butterfly(e[tt][2], e[tt][3], c2.x, -c2.y, 2 * t);
+        butterfly(e[tt][0], e[tt][2], c1.x, -c1.y, t);
+        butterfly(e[tt][1], e[tt][3], c9.x, -c9.y, t + 8);
+    }
+}
+
+// One block by the whole CTA.  Every thread reaches every barrier.  BUILD: the
+// CTA's tables are built here, while the pixel loads are in flight.
+template <int B, bool REUSE, bool BUILD>
+__device__ __forceinline__ void block(const ImageArgs& im, int by, int bx, const MethodArgs& mth, Smem* sm,
+                                      unsigned long long* empty, float delta) {
+    constexpr int PT = (B * B + T - 1) / T;   // target pixels per thread
+    const int tid = threadIdx.x, lane = tid & 31, q = tid >> 5;
+    const int L = mth.L, y0 = by * B - L, x0 = bx * B - L;
+    const long long blk = (long long)by * im.nbx + bx;
+    int16_t* seq = im.seq ? im.seq + (size_t)blk * im.K : nullptr;
+    const int q2 = ((q & 1) << 1) | (q >> 1);   // the two bits of q reversed
+
+    // ---- a1: 8 pixels of column `lane` per thread, and the target pixels ----
+    float f[8];
+    unsigned kn = 0, re = 0;
+    {
+        const int xc = x0 + lane;
+        const bool xin = (unsigned)xc < (unsigned)im.W;
+        const int pbx = xin ? xc / B : 0;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int y = y0 + in_index(q2, i);
+            bool known = false, reused = false;
+            float fv = 0.f, pv = 0.f;
+            if (xin && (unsigned)y < (unsigned)im.H) {
+                const size_t off = (size_t)y * im.pitch + xc;
+                known = __ldg(im.mask + off) != 0;
+                fv = __ldg(im.img + off);
+                if constexpr (REUSE) {
+                    const int pby = y / B;
+                    const bool earlier = pby < by || (pby == by && pbx < bx);
+                    // earlier targets were written by earlier launches: read through L2
+                    if (earlier) pv = __ldcg(im.out + off);
+                    reused = !known && earlier;
+                }
+            }
+            f[i] = known ? fv : (reused ? pv : 0.f);   // select: unknown values never enter arithmetic
+            kn |= known ? 1u << i : 0u;
+            re |= reused ? 1u << i : 0u;
+        }
+    }
+    float tv[PT];          // value of a known target pixel
+    bool tk[PT], tin[PT];  // known; in the image
+    unsigned need = 0;
+#pragma unroll
+    for (int p = 0; p < PT; ++p) {
+        const int i = tid + T * p;
+        const int ty = by * B + i / B, tx = bx * B + i % B;
+        tin[p] = i < B * B && ty < im.H && tx < im.W;
+        tk[p] = true;
+        tv[p] = 0.f;
+        if (tin[p]) {
+            const size_t off = (size_t)ty * im.pitch + tx;
+            tk[p] = __ldg(im.mask + off) != 0;
+            tv[p] = __ldg(im.img + off);
+        }
+        need |= tk[p] ? 0u : 2u;
+    }
+    if constexpr (BUILD) tables(mth, sm);
+    const unsigned avail = kn | re;
+    __syncthreads();   // the tables are complete, the buffers free
+    float wv[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int m = in_index(q2, i);
+        const float w0 = sm->w0[fold(m) * (S / 2) + fold(lane)];
+        // Eq. (5): w0 on known pixels, delta w0 on re-used ones, 0 elsewhere
+        wv[i] = ((kn >> i) & 1u) ? w0 : (((re >> i) & 1u) ? delta * w0 : 0.f);
+        sm->A[m * AS + lane] = make_float2(f[i], wv[i]);
+    }
+    need = __reduce_or_sync(FULL, need | (avail ? 1u : 0u));
+    if (lane == 0) sm->flags[q] = need;
+    __syncthreads();
+    need = sm->flags[0] | sm->flags[1] | sm->flags[2] | sm->flags[3];
+
+    float gacc[PT];
+#pragma unroll
+    for (int p = 0; p < PT; ++p) gacc[p] = 0.f;
+    const int K = im.K;
+    if (!(need & 1u)) {
+        if (tid == 0) empty_block(seq, K, empty);
+    } else if (K > 0) {
+        // ---- a2: sums over the column in row order, then over the columns
+        //      (every warp for itself: no barrier); weighted mean ----
+        float sw = 0.f, sfw = 0.f;
+#pragma unroll 8
+        for (int m = 0; m < S; ++m) {
+            const float2 fw = sm->A[m * AS + lane];
+            sw = __fadd_rn(sw, fw.y);
+            sfw = __fmaf_rn(fw.y, fw.x, sfw);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            sw += __shfl_xor_sync(FULL, sw, o);
+            sfw += __shfl_xor_sync(FULL, sfw, o);
+        }
+        const float mu = sfw / sw;
+        float2 x[8];
+        unsigned dmax = 0;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const bool av = (avail >> i) & 1u;
+            const float d = __fsub_rn(f[i], mu);
+            x[i] = make_float2(av ? __fmul_rn(d, wv[i]) : 0.f, wv[i]);
+            const unsigned ab = __float_as_uint(d) & 0x7fffffffu;
+            dmax = (av && ab > dmax) ? ab : dmax;
+        }
+        dmax = __reduce_max_sync(FULL, dmax);
+        if (lane == 0) sm->dmax[q] = dmax;
+        __syncthreads();
+        dmax = max(max(sm->dmax[0], sm->dmax[1]), max(sm->dmax[2], sm->dmax[3]));
+        unsigned aexp = (dmax >> 23) + 1u;             // exponent field of alpha = 2^e
+        aexp = (dmax >= 0x00800000u && dmax < 0x7e000000u) ? aexp : 127u;
+        const float alpha = __uint_as_float(aexp << 23);
+        const float inv2alpha = __uint_as_float((253u - aexp) << 23);   // 1 / (2 alpha)
+#pragma unroll
+        for (int i = 0; i < 8; ++i) x[i].y *= alpha;
+
+        // ---- a3: over the rows (lane n = column n), then over the columns (lane k = row k) ----
+#pragma unroll 1
+        for (int pass = 0; pass < 2; ++pass) {
+            float2 e[2][4];
+            fft32_split(x, e, sm->W, sm->cs, q, lane);
+            // first transform out by rows k, then back in by columns; the second stays transposed
+            const int sk = pass == 0 ? AS : 1, sl = pass == 0 ? 1 : AS;
+#pragma unroll
+            for (int tt = 0; tt < 2; ++tt)
+#pragma unroll
+                for (int p = 0; p < 4; ++p) sm->A[(2 * q + tt + 8 * p) * sk + lane * sl] = e[tt][p];
+            __syncthreads();
+            if (pass == 0) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) x[i] = sm->A[lane * AS + in_index(q2, i)];
+            }
+        }
+
+        // ---- Q and W of this thread's components ----
+        const int k = RPW * q + lane / G, g = lane % G;
+        float zr[NC], zi[NC], wf[NC], o[NC];
+        float2 wu[NC];   // the unshifted W row (DC phase)
+#pragma unroll
+        for (int j = 0; j < NC; ++j) {
+            const int l = g + G * j;
+            const float2 a = sm->A[k * AS + l], c = sm->A[((S - k) & (S - 1)) * AS + ((S - l) & (S - 1))];
+            wu[j] = make_float2((a.y + c.y) * inv2alpha, (c.x - a.x) * inv2alpha);
+            zr[j] = (a.x + c.x) * 0.5f;
+            zi[j] = (a.y - c.y) * 0.5f;
+            wf[j] = sm->wf[foldf(k) * H1 + foldf(l)];
+        }
+#pragma unroll
+        for (int j = 0; j < NC; ++j) {
+            float2* w = sm->W + k * WS + g + G * j;
+            w[0] = w[S] = w[S * WS] = w[S * WS + S] = wu[j];
+        }
+        __syncthreads();
+        const float cg = mth.gamma * (1.f / sm->W[0].x);
+        int pm[PT], pn[PT];
+#pragma unroll
+        for (int p = 0; p < PT; ++p) {
+            pm[p] = L + (tid + T * p) / B;
+            pn[p] = L + (tid + T * p) % B;
+        }
+        // W[k-u][l-v] lies u rows and v entries before this one
+        const float2* wbase = sm->W + (k + S) * WS + g + S;
+        const unsigned idx0 = (unsigned)(k * S + g);
+        int16_t* seq0 = tid == 0 ? seq : nullptr;
+        float cr = 0.f, ci = 0.f;
+        unsigned off;   // u * WS + v
+        float m;        // this thread's maximum
+        float2 csn[PT];
+#pragma unroll
+        for (int p = 0; p < PT; ++p) csn[p] = make_float2(0.f, 0.f);
+        // the last pick's share of the target pixels (sparse inverse of G)
+        auto target = [&]() {
+#pragma unroll
+            for (int p = 0; p < PT; ++p) gacc[p] = fma_rn(cr, csn[p].x, fma_rn(-ci, csn[p].y, gacc[p]));
+        };
+
+        // a5, a6 for the objectives o[] of the values (vr, vi): the warp's
+        // maximum (objectives are >= +0: their bits order like the values)
+        // and its lowest index, then the four warps' candidates.  What a
+        // thread would publish is formed while the reductions run.
+        auto pick = [&](int nu, const float (&vr)[NC], const float (&vi)[NC]) {
+            const unsigned mb = __float_as_uint(m);
+            const unsigned Mw = __reduce_max_sync(FULL, mb);
+            target();   // of the previous pick
+            unsigned jj[NC];
+#pragma unroll
+            for (int j = 0; j < NC; ++j) jj[j] = __float_as_uint(o[j]) == mb ? (unsigned)j : (unsigned)(NC - 1);
+            const unsigned bj = min(min(min(jj[0], jj[1]), min(jj[2], jj[3])), min(min(jj[4], jj[5]), min(jj[6], jj[7])));
+            const unsigned bidx = idx0 + G * bj;
+            const unsigned lo = __reduce_min_sync(FULL, mb == Mw ? bidx : (unsigned)(S * S));
+            float br = vr[NC - 1], bi = vi[NC - 1];
+#pragma unroll
+            for (int j = NC - 2; j >= 0; --j) {
+                const bool h = __float_as_uint(o[j]) == mb;
+                br = h ? vr[j] : br;
+                bi = h ? vi[j] : bi;
+            }
+            // c = gamma p (Eq. 10); index u * S + v as the offset u * WS + v
+            const float4 mine = make_float4(m, __uint_as_float((bidx >> 5) * WS + (bidx & (S - 1))), br * cg, bi * cg);
+            float4* sl = sm->slot[nu & 1];
+            if (mb == Mw && bidx == lo) sl[q] = mine;
+            __syncthreads();   // one barrier per iteration: the slots alternate
+            // rows ascend with the warp, so the first maximum has the lowest index
+            float4 c0 = sl[0], c2 = sl[2];
+            const float4 c1 = sl[1], c3 = sl[3];
+            if (__float_as_uint(c1.x) > __float_as_uint(c0.x)) c0 = c1;
+            if (__float_as_uint(c3.x) > __float_as_uint(c2.x)) c2 = c3;
+            if (__float_as_uint(c2.x) > __float_as_uint(c0.x)) c0 = c2;
+            off = __float_as_uint(c0.y);
+            cr = c0.z;
+            ci = c0.w;
+            const int u = (int)(off / WS), v = (int)(off % WS);
+            if (seq0 != nullptr) seq0[nu] = (int16_t)(u * S + v);
+#pragma unroll
+            for (int p = 0; p < PT; ++p) csn[p] = sm->cs[(u * pm[p] + v * pn[p]) & (S - 1)];
+        };
+        auto max_all = [&]() { m = max3(max3(o[0], o[1], o[2]), max3(o[3], o[4], o[5]), fmaxf(o[6], o[7])); };
+
+        // ---- a4-a8: the DC phase, R = a W + Q, then the plain loop ----
+        int nu = 0;
+        {
+            float ar = mu, ai = 0.f;
+            for (;;) {
+                float rr[NC], ri[NC];
+#pragma unroll
+                for (int j = 0; j < NC; ++j) {
+                    split_value(ar, ai, wu[j].x, wu[j].y, zr[j], zi[j], rr[j], ri[j]);
+                    o[j] = objective<float>(rr[j], ri[j], wf[j]);
+                }
+                max_all();
+                pick(nu, rr, ri);
+                if (++nu == K || off != 0) break;
+                ar -= cr;
+                ai -= ci;
+            }
+#pragma unroll
+            for (int j = 0; j < NC; ++j) split_value(ar, ai, wu[j].x, wu[j].y, zr[j], zi[j], zr[j], zi[j]);
+        }
+        while (nu < K) {
+            const float2* row = wbase - off;   // a7 (Eq. 12) and the next objective
+#pragma unroll
+            for (int j = 0; j < NC; ++j) {
+                const float2 w = row[G * j];
+                residual_update(zr[j], zi[j], w.x, w.y, cr, ci);
+                o[j] = objective<float>(zr[j], zi[j], wf[j]);
+            }
+            max_all();
+            pick(nu++, zr, zi);
+        }
+        target();
+    }
+
+    // ---- a9 ----
+#pragma unroll
+    for (int p = 0; p < PT; ++p) {
+        const int i = tid + T * p;
+        if (tin[p]) {
+            const int ty = by * B + i / B, tx = bx * B + i % B;
+            im.out[(size_t)ty * im.pitch + tx] = tk[p] ? tv[p] : gacc[p];
+        }
+    }
+}
+
+// One block per CTA, the grid sized to the work.  INLINE: one image whose
+// arguments are kernel parameters; else images and block prefix sums of a
+// work table in device memory.
+template <int B, bool INLINE>
+__global__ void __launch_bounds__(T) fsr_coop_kernel(const __grid_constant__ BatchArgs a,
+                                                     const __grid_constant__ ImageArgs one) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    Smem* sm = reinterpret_cast<Smem*>(smem);
+    const long long item = blockIdx.x;
+    if constexpr (INLINE) {
+        const int by = (int)item / one.nbx;
+        block<B, false, true>(one, by, (int)item - by * one.nbx, a.mth, sm, a.empty, 0.f);
+    } else {
+        int lo = 0, hi = a.n - 1;   // image of this entry: last i with first[i] <= item
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (__ldg(a.first + mid) <= item) lo = mid;
+            else hi = mid - 1;
+        }
+        const ImageArgs im = a.images[lo];
+        const int blk = (int)(item - __ldg(a.first + lo));
+        const int by = blk / im.nbx;
+        block<B, false, true>(im, by, blk - by * im.nbx, a.mth, sm, a.empty, 0.f);
+    }
+}
+
+// Re-use form: one launch per wavefront (see fsr_reuse_kernel), a CTA per block.
+template <int B, int NSEG>
+__global__ void __launch_bounds__(T) fsr_coop_reuse_kernel(const __grid_constant__ ReuseLaunchN<NSEG> a) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    Smem* sm = reinterpret_cast<Smem*>(smem);
+    tables(a.mth, sm);
+    // a programmatic dependent of the previous wavefront: nothing of the
+    // image or the output is read before that one has completed
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int j = blockIdx.x;
+    int s = 0;   // the segment (image) of block j
+    if constexpr (NSEG > 1) {
+        while (s + 1 < a.nseg && a.seg[s + 1].first <= j) ++s;
+    }
+    const ReuseSeg& sg = a.seg[s];
+    const int by = sg.by_lo + (j - sg.first);
+    block<B, true, false>(sg.im, by, a.t - a.slope * by, a.mth, sm, a.empty, a.delta);
+}
+
+}  // namespace coop
+}  // namespace fsrk

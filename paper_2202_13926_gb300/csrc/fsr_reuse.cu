@@ -1,7 +1,9 @@
 // Re-use of reconstructed pixels (the sequential form of the original FSR
 // that Sec. II leaves out): the wavefront kernel, FP32 and FP64, every B of
-// the 32 x 32 support.  One warp per block of the wavefront; the launch
-// shapes are in fsr_reuse.cuh.
+// the 32 x 32 support.  One warp per block of the wavefront (the launch
+// shapes are in fsr_reuse.cuh), or for FP32 wavefronts of few blocks a CTA
+// per block (fsr_coop.cuh): one 1080p frame, K = 100, delta = 0.5: 104.0 ->
+// 53.5 ms, six 480 x 270 frames 27.6 -> 14.7 ms, bit-identical.
 #include "fsr_reuse.cuh"
 
 namespace fsrk {
@@ -16,6 +18,7 @@ cudaError_t configure_reuse() {
 cudaError_t launch_reuse(const ReuseLaunch& a, int B, int fp64, int sm_count, cudaStream_t stream) {
     if (a.total <= 0) return cudaSuccess;
     if (fp64) return launch_reuse_f64(a, B, sm_count, stream);
+    if (a.total <= (long long)kCoopReusePerSm * sm_count) return launch_coop_reuse(a, B, stream);
     if (B == 2 || B == 4) return launch_reuse_f32lo(a, B, sm_count, stream);
     return launch_reuse_f32hi(a, B, sm_count, stream);
 }

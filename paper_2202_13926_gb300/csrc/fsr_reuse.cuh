@@ -10,14 +10,12 @@
 namespace fsrk {
 namespace reuse {
 
-// Warps per CTA of the FP32 wavefront kernel.  A wavefront of one image
-// holds at most (blocks per image row) / (ceil(L / B) + 1) blocks (96 on a
-// 1080p frame at B = 4), far fewer than the SMs can hold, so the per-block
-// latency sets the time: small CTAs spread the blocks over more SMs (1080p,
-// K = 100, delta = 0.5: 145 ms per frame with 8 warps per CTA, 130 ms with 1,
-// 119 ms with 2, 115 ms with 4).  A launch holding the wavefronts of many
-// images takes CTAs of 8 warps once its blocks exceed what CTAs of 4 hold in
-// one wave (3 per SM by shared memory, against 2 CTAs of 8 = 16 warps).
+// Warps per CTA.  FP64: a wavefront of one image holds at most (blocks per
+// image row) / (ceil(L / B) + 1) blocks (96 on a 1080p frame at B = 4), far
+// fewer than the SMs can hold, so small CTAs spread them over more SMs.  FP32
+// comes here with the wavefronts of many images (more than kCoopReusePerSm
+// blocks per SM): CTAs of 4 warps while the blocks fit one wave of them (3
+// per SM by shared memory), of 8 beyond (2 CTAs of 8 = 16 warps per SM).
 constexpr int kWarpsReuse = 4;
 constexpr int kWarpsReuseWide = 8;
 constexpr int kCtasPerSmReuse = 3;
@@ -32,7 +30,8 @@ cudaError_t configure_one() {
 // may start (and build their tables) while the previous wavefront runs; the
 // kernel waits for that wavefront's completion before it reads any pixel.
 // 1080p, K = 100, delta = 0.5, 4 warps per CTA: 115.8 ms per frame with
-// plain stream order, 103.8 ms with this launch (outputs bit-identical).
+// plain stream order, 103.8 ms with this launch (outputs bit-identical; one
+// warp per block, which this frame no longer takes).
 template <typename T, int B, int WARPS, int NSEG>
 cudaError_t launch_one(const ReuseLaunchN<NSEG>& a, cudaStream_t stream) {
     cudaLaunchConfig_t cfg = {};
@@ -48,15 +47,14 @@ cudaError_t launch_one(const ReuseLaunchN<NSEG>& a, cudaStream_t stream) {
     return cudaLaunchKernelEx(&cfg, fsr_reuse_kernel<T, B, WARPS, NSEG>, a);
 }
 
-// instantiated forms: one image in CTAs of 4 warps; up to kReuseSegs images
-// in CTAs of 4, or of 8 for FP32 launches beyond one wave of CTAs of 4
+// instantiated forms: up to kReuseSegs images in CTAs of 4 warps; FP32 also
+// in CTAs of 8, FP64 also with one image's parameters alone
 template <typename T, int B>
 cudaError_t configure_b() {
     cudaError_t e;
-    if ((e = configure_one<T, B, kWarpsReuse, 1>()) != cudaSuccess) return e;
     if ((e = configure_one<T, B, kWarpsReuse, kReuseSegs>()) != cudaSuccess) return e;
     if constexpr (sizeof(T) == 4) return configure_one<T, B, kWarpsReuseWide, kReuseSegs>();
-    return cudaSuccess;
+    else return configure_one<T, B, kWarpsReuse, 1>();
 }
 
 template <typename T, int B>
@@ -64,8 +62,9 @@ cudaError_t launch_b(const ReuseLaunch& a, int sm_count, cudaStream_t stream) {
     if constexpr (sizeof(T) == 4) {
         if (a.total > kCtasPerSmReuse * kWarpsReuse * sm_count)
             return launch_one<T, B, kWarpsReuseWide, kReuseSegs>(a, stream);
+    } else {
+        if (a.nseg == 1) return launch_one<T, B, kWarpsReuse, 1>(one_image(a), stream);
     }
-    if (a.nseg == 1) return launch_one<T, B, kWarpsReuse, 1>(one_image(a), stream);
     return launch_one<T, B, kWarpsReuse, kReuseSegs>(a, stream);
 }
 
