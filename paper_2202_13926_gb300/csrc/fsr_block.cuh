@@ -78,6 +78,7 @@ struct TileMaps {
 
 // Device status word bits (set by kernels, read and cleared by the host).
 constexpr unsigned kStatusTileWait = 1u;   // a bounded wait on a tile copy gave up
+constexpr unsigned kStatusRowWait = 4u;    // a bounded wait of the re-use form for the row above gave up
 
 // Single image: warps take blocks one at a time from a device work counter.
 struct KernelArgs {
@@ -588,7 +589,11 @@ __device__ __forceinline__ void residual_update(T& re, T& im, T wr, T wi, T cr, 
 // maximum.
 
 constexpr int WS32 = WRow<float>::stride;
-constexpr int NG = 2;            // groups per row
+// Groups per row: the group holding the maximum is published, so more groups
+// mean fewer stores and more to search.  1080p, K = 100, ms per frame with the
+// pick by reductions: 2 groups 4.82, 4 groups 4.65, 8 groups 4.78 (2 groups
+// and ballots: 4.84).
+constexpr int NG = 4;            // groups per row
 constexpr int GS = S / NG;       // components per group
 static_assert(GS % 4 == 0 && GS <= 16, "a group is published as GS / 4 float4 stores");
 
@@ -771,20 +776,13 @@ __device__ __forceinline__ Pick argmax_pick(const float (&zr)[S], const float (&
                                             float ar, float ai, int lane) {
     const float m = groups_max(g);
     const unsigned Mb = __reduce_max_sync(FULL, __float_as_uint(m));
-    const unsigned bu = __ballot_sync(FULL, __float_as_uint(m) == Mb);
-    const int u = __ffs(bu) - 1;
-    // first group of lane u's row that holds the maximum
-    int jg;
-    if constexpr (NG == 2) {
-        // a second ballot, independent of u: bit u says whether group 0 holds it
-        const unsigned b0 = __ballot_sync(FULL, __float_as_uint(g[0]) == Mb);
-        jg = ((b0 >> u) & 1u) ? 0 : 1;
-    } else {
-        jg = NG - 1;
+    // the lowest (row, group of the row) holding it, by a second reduction: a
+    // ballot costs a find-first-set, which is slower than the reduction
+    unsigned c0 = 64u * NG;
 #pragma unroll
-        for (int j = NG - 2; j >= 0; --j) jg = (__float_as_uint(g[j]) == Mb) ? j : jg;
-        jg = __shfl_sync(FULL, jg, u);
-    }
+    for (int j = NG - 1; j >= 0; --j) c0 = __float_as_uint(g[j]) == Mb ? (unsigned)(NG * lane + j) : c0;
+    const unsigned cm = __reduce_min_sync(FULL, c0);
+    const int u = (int)(cm / NG) & (S - 1), jg = (int)(cm % NG);
     publish_group(zr, zi, jg, lane == u, rowbuf);
     __syncwarp();
     const int cl = GS * jg + (lane & (GS - 1));   // column examined by this lane
@@ -795,7 +793,7 @@ __device__ __forceinline__ Pick argmax_pick(const float (&zr)[S], const float (&
         split_value(ar, ai, w.x, w.y, q.x, q.y, rr, ri);
     }
     const float o = objective<float>(rr, ri, swf[u * WFS + cl]);
-    const int vl = __ffs(__ballot_sync(FULL, __float_as_uint(o) == Mb)) - 1;   // lanes 0..GS-1 lead
+    const int vl = (int)__reduce_min_sync(FULL, __float_as_uint(o) == Mb ? (unsigned)(lane & (GS - 1)) : GS - 1u);
     Pick pk;
     pk.u = u;
     pk.v = GS * jg + vl;
@@ -1175,8 +1173,70 @@ fsr_blocks_kernel(const __grid_constant__ KernelArgs a) {
     }
 }
 
-// Batch form: every warp takes `chunk` consecutive entries of the block list
-// at a time; images are ordered by decreasing K so the long blocks start first.
+// ---- work list of the batch form --------------------------------------------
+
+// Image of an entry of the block list: the last i with first[i] <= item.
+__device__ __forceinline__ int image_of(const BatchArgs& a, long long item) {
+    int lo = 0, hi = a.n - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (__ldg(a.first + mid) <= item) lo = mid;
+        else hi = mid - 1;
+    }
+    return lo;
+}
+
+constexpr int kTakeShare = 8;
+
+// Entries a warp takes at once: a share of what is left (so that the warps
+// end together), at least `least` and at most 32 (one scan of a lane each).
+__device__ __forceinline__ int guided_take(const BatchArgs& a, long long seen, int warps, int least) {
+    const long long left = a.total - seen;
+    const unsigned share = (unsigned)(left < 0x7fffffffll ? left : 0x7fffffffll) / (unsigned)(kTakeShare * warps);
+    return max(least, (int)min(share, 32u));
+}
+
+// Entries base .. base + count - 1 (count <= 32), one per lane: a block whose
+// target pixels are all known is its input copied, whatever the model (end of
+// Sec. II), so its lane copies it here and the block is done (4K, one 16 x 16
+// macroblock in ten lost, S = 32, K = 50: 10.39 -> 1.42 ms).  Returns the
+// entries that need the iteration: those with an unknown target pixel, and
+// those whose selected indices are asked for.
+template <int B>
+__device__ __forceinline__ unsigned scan_targets(const BatchArgs& a, long long base, int count, int lane) {
+    const long long item = base + lane;
+    bool need = false;
+    if (lane < count && item < a.total) {
+        const int lo = image_of(a, item);
+        const ImageArgs* im = a.images + lo;
+        const int blk_x = im->nbx, W = im->W, H = im->H, pitch = im->pitch;
+        const long long blk = item - __ldg(a.first + lo);
+        const int by = (int)(blk / blk_x), bx = (int)(blk - (long long)by * blk_x);
+        const int rows = min(B, H - by * B), cols = min(B, W - bx * B);
+        const size_t off = (size_t)by * B * pitch + (size_t)bx * B;
+        const uint8_t* mask = im->mask + off;
+        need = im->seq != nullptr;
+        for (int r = 0; r < rows && !need; ++r) {
+            unsigned known = 1;
+#pragma unroll
+            for (int c = 0; c < B; ++c)
+                if (c < cols) known = __ldg(mask + (size_t)r * pitch + c) != 0 ? known : 0u;
+            need = known == 0;
+        }
+        if (!need) {
+            const float* img = im->img + off;
+            float* out = im->out + off;
+            for (int r = 0; r < rows; ++r)
+#pragma unroll
+                for (int c = 0; c < B; ++c)
+                    if (c < cols) out[(size_t)r * pitch + c] = __ldg(img + (size_t)r * pitch + c);
+        }
+    }
+    return __ballot_sync(FULL, need);
+}
+
+// Batch form: every warp takes consecutive entries of the block list
+// (guided_take) at a time; images are ordered by decreasing K so the long blocks start first.
 // ONE_ROUND: short-lived CTAs (a warp takes one chunk; the grid is sized to
 // the work), used by the serving loop so that the CTAs of a launch on a
 // higher-priority stream are scheduled as soon as running CTAs finish.
@@ -1208,30 +1268,31 @@ fsr_batch_kernel(const BatchArgs a) {
     }
 
     const T gamma = T(a.mth.gamma);
+    long long seen = 0;   // entries taken by all warps, as of this warp's last take
     for (;;) {
+        const int take = ONE_ROUND ? a.chunk : guided_take(a, seen, (int)gridDim.x * WARPS, a.chunk);
         unsigned long long base = 0;
-        if (lane == 0) base = atomicAdd(a.counter, (unsigned long long)a.chunk);
+        if (lane == 0) base = atomicAdd(a.counter, (unsigned long long)take);
         base = __shfl_sync(FULL, base, 0);
         if (base >= (unsigned long long)a.total) break;
-        const long long end = min((long long)base + a.chunk, a.total);
+        seen = (long long)base;
         bool ok = true;
-        for (long long item = (long long)base; item < end && ok; ++item) {
-            // image of this entry: last i with first[i] <= item
-            int lo = 0, hi = a.n - 1;
-            while (lo < hi) {
-                const int mid = (lo + hi + 1) >> 1;
-                if (__ldg(a.first + mid) <= item) lo = mid;
-                else hi = mid - 1;
+        for (int sub = 0; sub < take && ok; sub += 32) {
+            unsigned todo = scan_targets<B>(a, seen + sub, min(take - sub, 32), lane);
+            while (todo != 0 && ok) {
+                const long long item = seen + sub + (__ffs(todo) - 1);
+                todo &= todo - 1;
+                const int lo = image_of(a, item);
+                const ImageArgs im = a.images[lo];
+                TileReq tr;
+                tr.maps = (tiles && im.tiles) ? a.maps + lo : nullptr;
+                tr.status = a.status;
+                tr.bytes = kTileBytes + (unsigned)a.tx_extra;
+                tr.bar = smem_addr(smem + Lay::bar_off(WARPS) + 8 * warp);
+                tr.parity = reinterpret_cast<uint32_t*>(smem + Lay::parity_off(WARPS)) + warp;
+                ok = process_block<T, B, CONJ>(im, item - __ldg(a.first + lo), a.mth.L, gamma, sw0, swf, scs, Wd,
+                                               rowbuf, tr, a.empty, lane);
             }
-            const ImageArgs im = a.images[lo];
-            TileReq tr;
-            tr.maps = (tiles && im.tiles) ? a.maps + lo : nullptr;
-            tr.status = a.status;
-            tr.bytes = kTileBytes + (unsigned)a.tx_extra;
-            tr.bar = smem_addr(smem + Lay::bar_off(WARPS) + 8 * warp);
-            tr.parity = reinterpret_cast<uint32_t*>(smem + Lay::parity_off(WARPS)) + warp;
-            ok = process_block<T, B, CONJ>(im, item - __ldg(a.first + lo), a.mth.L, gamma, sw0, swf, scs, Wd,
-                                           rowbuf, tr, a.empty, lane);
         }
         if (!ok) break;   // a tile wait gave up: this warp takes no more blocks
         if constexpr (ONE_ROUND) break;

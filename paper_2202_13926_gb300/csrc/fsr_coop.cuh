@@ -223,7 +223,7 @@ __device__ __forceinline__ void block(const ImageArgs& im, int by, int bx, const
     const int K = im.K;
     if (!(need & 1u)) {
         if (tid == 0) empty_block(seq, K, empty);
-    } else if (K > 0) {
+    } else if (K > 0 && ((need & 2u) || seq != nullptr)) {   // all targets known: copied, whatever the model
         // ---- a2: sums over the column in row order, then over the columns
         //      (every warp for itself: no barrier); weighted mean ----
         float sw = 0.f, sfw = 0.f;

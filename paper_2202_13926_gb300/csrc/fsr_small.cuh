@@ -792,6 +792,7 @@ __device__ __forceinline__ void run(const BatchArgs& a) {
                 else hi = mid - 1;
             }
             const ImageArgs im = a.images[lo];
+            if (scan_targets<B>(a, item, 1, lane) == 0u) continue;   // all targets known: copied
             block<T, SZ, B>(im, item - __ldg(a.first + lo), a.mth.L, gamma, sw0, swf, stw, stt, area, a.empty,
                             lane);
         }
