@@ -1,5 +1,5 @@
-// FP32 FSR with a support S in {4, 8, 16} (B <= S; the support-size study of
-// Sec. IV, Figs. 3 and 5): one group of S lanes per block, 32 / S blocks per
+// FP32 FSR with a support S in {8, 16} (B <= S; the support-size study of Sec.
+// IV, Figs. 3 and 5; S = 4: fsr_quad.cu): one group of S lanes per block, 32 / S blocks per
 // warp.  Lane t of a group holds column t of the support, then row t of the
 // spectrum (S complex values in registers), as the S = 32 kernel does with a
 // whole warp:
@@ -32,7 +32,7 @@ namespace {
 
 template <int SZ>
 struct Grp {
-    static_assert(SZ == 4 || SZ == 8 || SZ == 16, "group kernels cover S = 4, 8, 16");
+    static_assert(SZ == 8 || SZ == 16, "group kernels cover S = 8 and 16");
     static constexpr int WS = 2 * SZ + 1;            // W row stride (float2)
     static constexpr int TS = SZ + 1;                // transpose stride (float2)
     static constexpr int WFS = SZ + 1;               // w_f row stride (float)
@@ -49,8 +49,8 @@ struct Grp {
     static constexpr size_t wf_off = w0_off + 4 * SZ * SZ;
     // w_f again with one copy per group of a warp side by side in 32-word
     // rows: group g reads its copy at words 32 u + S g + t, on banks no other
-    // group of the warp touches, whatever row u it picked (1080p: S = 8
-    // 0.702 -> 0.683 ms, S = 16 1.797 -> 1.776 ms)
+    // group of the warp touches, whatever row u it picked (1080p: S = 8 0.702
+    // -> 0.683 ms, S = 16 1.797 -> 1.776 ms)
     static constexpr size_t wfg_off = wf_off + 4 * SZ * WFS;
     static constexpr size_t cs_off = wfg_off + 4 * SZ * 32;
     static constexpr size_t warp0_off = (cs_off + 8 * SZ + 127) & ~(size_t)127;
@@ -116,6 +116,27 @@ __device__ __forceinline__ unsigned group_umax(unsigned v) {
 #pragma unroll
     for (int s = SZ / 2; s > 0; s >>= 1) v = max(v, (unsigned)__shfl_xor_sync(FULL, v, s));
     return v;
+}
+// per-group maximum / minimum by one full-warp reduction per group
+template <int SZ>
+__device__ __forceinline__ unsigned group_rmax(unsigned v, int grp) {
+    unsigned r = 0;
+#pragma unroll
+    for (int g = 0; g < 32 / SZ; ++g) {
+        const unsigned x = __reduce_max_sync(FULL, grp == g ? v : 0u);
+        r = grp == g ? x : r;
+    }
+    return r;
+}
+template <int SZ>
+__device__ __forceinline__ unsigned group_rmin(unsigned v, int grp) {
+    unsigned r = 0;
+#pragma unroll
+    for (int g = 0; g < 32 / SZ; ++g) {
+        const unsigned x = __reduce_min_sync(FULL, grp == g ? v : 0xffffffffu);
+        r = grp == g ? x : r;
+    }
+    return r;
 }
 template <int SZ>
 __device__ __forceinline__ float group_sum(float v) {
@@ -186,6 +207,24 @@ __device__ __forceinline__ void group_block(const ImageArgs& im, long long blk, 
             }
         }
         zr[m] = f;   // unknown values never enter arithmetic
+    }
+    int16_t* seq = (valid && im.seq) ? im.seq + (size_t)blk * im.K : nullptr;
+    // A target whose pixels are all known is its input copied, whatever the
+    // model (end of Sec. II): nothing to iterate when that holds for every
+    // block of the warp (and no selected indices are asked for).
+    const unsigned rows_in = valid ? (unsigned)min(B, im.H - by * B) : 0u;   // target rows in the image
+    const bool fill = (unsigned)(t - L) < (unsigned)B && x < im.W && ((~known >> L) & ((1u << rows_in) - 1u)) != 0u;
+    if (!__any_sync(FULL, fill || seq != nullptr)) {
+#pragma unroll
+        for (int q = 0; q < PT; ++q) {
+            const int pidx = t + SZ * q;
+            const int ty = by * B + pidx / B, tx = bx * B + pidx % B;
+            if (valid && pidx < B * B && ty < im.H && tx < im.W) {
+                const size_t off = (size_t)ty * im.pitch + tx;
+                im.out[off] = __ldg(im.img + off);
+            }
+        }
+        return;
     }
     float sw = 0.f, sfw = 0.f;
 #pragma unroll
@@ -281,7 +320,6 @@ __device__ __forceinline__ void group_block(const ImageArgs& im, long long blk, 
         gacc[q] = 0.f;
     }
     const int Kh = valid ? im.K : 0;
-    int16_t* seq = (valid && im.seq) ? im.seq + (size_t)blk * im.K : nullptr;
     if (valid && !active && t == 0) empty_block(seq, im.K, empty);
     const float cg = active ? gamma * (1.f / W0) : 0.f;   // c = R[u,v] gamma / W[0,0] (Eqs. 10, 11)
     bool split = true;             // R = a W + Q (DC phase)
@@ -297,12 +335,21 @@ __device__ __forceinline__ void group_block(const ImageArgs& im, long long blk, 
         const int Kr = all ? Kmax : Kh;
         // a5: block maximum (each group reduces over its own lanes), the
         // lowest row holding it, then its lowest column
-        // (a butterfly over the group's lanes: a warp reduction with the
-        // group's lane mask runs once per group; 1080p: S = 4 0.366 -> 0.270
-        // ms, S = 8 0.718 -> 0.705 ms, S = 16 1.842 -> 1.798 ms)
-        const unsigned Mb = group_umax<SZ>(run ? __float_as_uint(m_lane) : 0u);
-        const unsigned ub = (__ballot_sync(FULL, run && __float_as_uint(m_lane) == Mb) >> gb) & G::LOW;
-        const int u = ub ? __ffs(ub) - 1 : 0;
+        // (one full-warp reduction per group, the other groups' lanes put in
+        // neutral values: 40 cycles for two groups where a shuffle butterfly
+        // takes 120; a ballot costs a find-first-set, for two groups more than
+        // two reductions and for four less.  64 x 64 image, K = 100: S = 16
+        // 73.6 -> 66.6 us, S = 8 56.4 -> 48.7 us; 1080p: S = 16 1.77 -> 1.75 ms,
+        // S = 8 670 -> 653 us)
+        const unsigned Mb = group_rmax<SZ>(run ? __float_as_uint(m_lane) : 0u, lane / SZ);
+        const bool hit = run && __float_as_uint(m_lane) == Mb;
+        int u;
+        if constexpr (SZ == 16) {
+            u = (int)group_rmin<SZ>(hit ? (unsigned)t : SZ - 1u, lane / SZ);
+        } else {
+            const unsigned ub = (__ballot_sync(FULL, hit) >> gb) & G::LOW;
+            u = ub ? __ffs(ub) - 1 : 0;
+        }
         __syncwarp();   // the previous pick's reads of the published row are done
         if (run && t == u) {
             float4* pub = reinterpret_cast<float4*>(rowbuf);
@@ -361,12 +408,11 @@ __device__ __forceinline__ void group_block(const ImageArgs& im, long long blk, 
         }
     };
     // the loops run to the largest K of the warp (uniform): a DC loop, then a
-    // loop without the split branches (1080p frame: S = 4 0.385 -> 0.365 ms,
-    // S = 8 0.776 -> 0.747 ms; S = 16 at 20 warps per SM 1.935 -> 1.922 ms,
-    // at 16 warps and 123 registers 2.07 -> 2.15 ms), in a form without the
+    // loop without the split branches (1080p frame: S = 8 0.776 -> 0.747 ms;
+    // S = 16 at 20 warps per SM 1.935 -> 1.922 ms), in a form without the
     // per-group run conditions when every group runs to the same K (S = 16
-    // 1.902 -> 1.848 ms, S = 4 0.369 -> 0.358 ms; S = 8 unchanged, with 32
-    // bytes spilled, so it keeps one form)
+    // 1.902 -> 1.848 ms; S = 8 unchanged, with 32 bytes spilled at the time, so
+    // it keeps one form)
     int nu = 0;
     while (nu < Kmax && __any_sync(FULL, split && active && nu < Kh)) step(nu++, true, false);
     if constexpr (SZ != 8) {
@@ -392,15 +438,20 @@ __device__ __forceinline__ void group_block(const ImageArgs& im, long long blk, 
     }
 }
 
-// Warps per CTA and CTAs per SM the register budget is set for: 20 warps
-// per SM at S = 16 (2 x 10, <= 96 registers, no spill), 32 at S = 8 (4 x 8,
-// <= 64, 36 bytes spilled) and at S = 4 (4 x 8, <= 64, no spill).  Measured
-// on the 1080p frame, K = 100: S = 4 0.53 ms with 16 warps per SM, 0.39 ms
-// with 32; S = 8 0.91 ms with 16, 0.745 ms with 24 (3 x 8), 0.722 ms with
-// 32; S = 16 2.07 ms with 16 (2 x 8), 1.93 ms with 20 (2 x 10 or 4 x 5),
-// 2.19 ms with 21 (3 x 7), 2.13 ms with 24 (2 x 12, 52 bytes spilled).
+// Warps per CTA and CTAs per SM the register budget is set for: 20 warps per SM
+// at S = 16 (2 x 10, <= 96 registers), 24 at S = 8 (3 x 8, <= 80).  Measured on
+// the 1080p frame, K = 100: S = 8 653 us with 24 warps, 659 with 32 (4 x 8, <=
+// 64, 40 bytes spilled; and a 256 x 256 image 62 instead of 50 us), 668 with 28;
+// S = 16 2.07 ms with 16 (2 x 8), 1.93 ms with 20 (2 x 10 or 4 x 5), 2.19 ms
+// with 21 (3 x 7), 2.13 ms with 24 (2 x 12, 52 bytes spilled) at the time.
+//
+// Tried for S = 8 and 16 and not kept: rows in packed pairs as in fsr_quad.cu
+// (91 instead of 121 instructions per block-iteration at S = 16, but 16-byte W
+// entries leave 16 warps per SM, and the pick's latency shows: 1.90 ms per
+// 1080p frame with a row per lane, 2.06 with two; S = 8 with two rows per lane
+// 555 us per 1080p frame, but 86 instead of 56 us for small images).
 template <int SZ> constexpr int group_warps() { return SZ == 16 ? 10 : 8; }
-template <int SZ> constexpr int group_min_ctas() { return SZ == 16 ? 2 : 4; }
+template <int SZ> constexpr int group_min_ctas() { return SZ == 16 ? 2 : 3; }
 
 template <int SZ, int B, int WARPS>
 __global__ void __launch_bounds__(WARPS * 32, group_min_ctas<SZ>()) fsr_group_kernel(const BatchArgs a) {
@@ -501,20 +552,16 @@ cudaError_t configure_group() {
     if ((e = configure_one<16, 4>()) != cudaSuccess) return e;
     if ((e = configure_one<16, 8>()) != cudaSuccess) return e;
     if ((e = configure_one<8, 2>()) != cudaSuccess) return e;
-    if ((e = configure_one<8, 4>()) != cudaSuccess) return e;
-    if ((e = configure_one<4, 2>()) != cudaSuccess) return e;
-    return configure_one<4, 4>();
+    return configure_one<8, 4>();
 }
 
-// FP32, S in {4, 8, 16}
+// FP32, S in {8, 16}
 cudaError_t launch_group(const BatchArgs& a, int S, int B, int chunk, int sm_count, cudaStream_t stream) {
     if (S == 16 && B == 2) return launch_one<16, 2>(a, chunk, sm_count, stream);
     if (S == 16 && B == 4) return launch_one<16, 4>(a, chunk, sm_count, stream);
     if (S == 16 && B == 8) return launch_one<16, 8>(a, chunk, sm_count, stream);
     if (S == 8 && B == 2) return launch_one<8, 2>(a, chunk, sm_count, stream);
     if (S == 8 && B == 4) return launch_one<8, 4>(a, chunk, sm_count, stream);
-    if (S == 4 && B == 2) return launch_one<4, 2>(a, chunk, sm_count, stream);
-    if (S == 4 && B == 4) return launch_one<4, 4>(a, chunk, sm_count, stream);
     return cudaErrorNotSupported;
 }
 

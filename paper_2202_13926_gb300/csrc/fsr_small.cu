@@ -1,5 +1,6 @@
-// Dispatch of the supports smaller than 32.  FP32 at S = 4, 8, 16 runs the
-// group kernel of fsr_group.cu (a group of S lanes per block); S = 24 (FP32
+// Dispatch of the supports smaller than 32.  FP32 at S = 8 and 16 runs the
+// group kernel of fsr_group.cu (a group of S lanes per block), at S = 4 the
+// kernel of fsr_quad.cu (a lane per block); S = 24 (FP32
 // and FP64) runs the lane-patch kernel of fsr_small.cuh, instantiated in
 // fsr_small24.cu; FP64 at S = 8 and 16 runs the same lane-patch kernel
 // (instantiated here) and FP64 at S = 4 the half-warp kernel of fsr_tiny.cu.
@@ -12,6 +13,8 @@ cudaError_t launch_small24(const BatchArgs& a, int B, int fp64, int chunk, int s
 cudaError_t launch_tiny(const BatchArgs& a, int B, int chunk, int sm_count, cudaStream_t stream);
 cudaError_t configure_group();
 cudaError_t launch_group(const BatchArgs& a, int S, int B, int chunk, int sm_count, cudaStream_t stream);
+cudaError_t configure_quad();
+cudaError_t launch_quad(const BatchArgs& a, int B, int chunk, int sm_count, cudaStream_t stream);
 
 namespace {
 
@@ -47,13 +50,15 @@ cudaError_t configure_small() {
     cudaError_t e = configure_patch_small();
     if (e != cudaSuccess) return e;
     if ((e = configure_group()) != cudaSuccess) return e;
+    if ((e = configure_quad()) != cudaSuccess) return e;
     return configure_small24();
 }
 
 cudaError_t launch_batch_small(const BatchArgs& a, int S, int B, int fp64, int chunk, int sm_count,
                                cudaStream_t stream) {
     if (S == 24) return launch_small24(a, B, fp64, chunk, sm_count, stream);
-    if (!fp64 && (S == 4 || S == 8 || S == 16)) return launch_group(a, S, B, chunk, sm_count, stream);
+    if (!fp64 && (S == 8 || S == 16)) return launch_group(a, S, B, chunk, sm_count, stream);
+    if (!fp64 && S == 4) return launch_quad(a, B, chunk, sm_count, stream);
     if (fp64 && S == 4) return launch_tiny(a, B, chunk, sm_count, stream);
     if (!fp64) return cudaErrorNotSupported;
     return launch_patch_small(a, S, B, chunk, sm_count, stream);
