@@ -207,8 +207,9 @@ int read_status(fsr_handle* h) {
     if ((e = cudaMemset(h->d_status, 0, sizeof st)) != cudaSuccess)
         return fail(h, FSR_ERR_CUDA, "clearing the status word: %s", cudaGetErrorString(e));
     return fail(h, FSR_ERR_TIMEOUT,
-                "status 0x%x: a kernel's bounded wait for a support-tile copy gave up; the warps concerned "
-                "stopped and their remaining blocks were not written",
+                "status 0x%x: a kernel's bounded wait (1: for a support-tile copy, 2: for a tensor-core pass, 4: for "
+                "the block row above) gave up; the warps concerned stopped and their remaining blocks were not "
+                "written",
                 st);
 }
 
@@ -276,8 +277,39 @@ int enqueue_single_fp32(fsr_handle* h, const float* img, const uint8_t* mask, in
 // and share the launches: launch t holds wavefront t of every image that has
 // one (up to kReuseSegs images per launch; more images take more launches
 // for the same t).
+//
+// FP32 with few enough rows at work runs in one launch instead, whose block
+// rows follow each other by progress flags (enqueue_reuse_rows).  Not while
+// the stream is being captured: the flags live in the handle's slots, which a
+// replayed graph would share with later calls.
+int enqueue_reuse_rows(fsr_handle* h, int n, const fsrk::ImageArgs* ims, const fsr_params* p, cudaStream_t stream) {
+    const int slot = (int)(h->row_next++ % fsr_handle::kRowSlots);
+    void* ring = static_cast<char*>(h->d_rows) + (size_t)slot * ((fsrk::coop_rows_bytes() + 255) & ~(size_t)255);
+    cudaError_t e = h->row_used[slot] ? cudaStreamWaitEvent(stream, h->row_ev[slot], 0) : cudaSuccess;
+    if (e == cudaSuccess)
+        e = fsrk::launch_coop_rows(method_args(p), p->reuse, n, ims, ring, h->d_status, h->d_empty, p->block,
+                                   h->sm_count, stream);
+    const cudaError_t er = cudaEventRecord(h->row_ev[slot], stream);
+    if (er == cudaSuccess) h->row_used[slot] = true;
+    if (e == cudaSuccess) e = er;
+    if (e != cudaSuccess) return fail(h, FSR_ERR_CUDA, "re-use launch failed: %s", cudaGetErrorString(e));
+    return ok(h);
+}
+
+bool not_capturing(cudaStream_t stream) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(stream, &st) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return st == cudaStreamCaptureStatusNone;
+}
+
 int enqueue_reuse_images(fsr_handle* h, int n, const fsrk::ImageArgs* ims, const fsr_params* p,
                          cudaStream_t stream) {
+    if (p->precision == FSR_FP32 &&
+        fsrk::coop_rows_parallel(n, ims, p->border, p->block) <= (long long)fsrk::kCoopRowsPerSm * h->sm_count && not_capturing(stream))
+        return enqueue_reuse_rows(h, n, ims, p, stream);
     fsrk::ReuseLaunch a;
     std::memset(&a, 0, sizeof a);
     a.mth = method_args(p);
@@ -587,8 +619,15 @@ int fsr_create(const fsr_config* cfg, fsr_handle** out) {
         bool okay = cudaMalloc(&h->d_single, sb) == cudaSuccess && cudaMallocHost(&h->h_single, sb) == cudaSuccess;
         for (int i = 0; okay && i < fsr_handle::kSingleSlots; ++i)
             okay = cudaEventCreateWithFlags(&h->single_ev[i], cudaEventDisableTiming) == cudaSuccess;
+        const size_t rb = ((fsrk::coop_rows_bytes() + 255) & ~(size_t)255) * fsr_handle::kRowSlots;
+        okay = okay && cudaMalloc(&h->d_rows, rb) == cudaSuccess;
+        for (int i = 0; okay && i < fsr_handle::kRowSlots; ++i)
+            okay = cudaEventCreateWithFlags(&h->row_ev[i], cudaEventDisableTiming) == cudaSuccess;
         if (!okay) {
             cudaGetLastError();
+            for (cudaEvent_t ev : h->row_ev)
+                if (ev) cudaEventDestroy(ev);
+            cudaFree(h->d_rows);
             for (cudaEvent_t ev : h->single_ev)
                 if (ev) cudaEventDestroy(ev);
             cudaFree(h->d_single);
@@ -623,8 +662,11 @@ int fsr_destroy(fsr_handle* h) {
             cudaFree(h->d_table);
             cudaFree(h->d_status);
             cudaFree(h->d_single);
+            cudaFree(h->d_rows);
             if (h->h_single) cudaFreeHost(h->h_single);
             for (cudaEvent_t ev : h->single_ev)
+                if (ev) cudaEventDestroy(ev);
+            for (cudaEvent_t ev : h->row_ev)
                 if (ev) cudaEventDestroy(ev);
             if (h->h_table) cudaFreeHost(h->h_table);
             if (h->table_free) cudaEventDestroy(h->table_free);

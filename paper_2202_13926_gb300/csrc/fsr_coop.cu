@@ -1,4 +1,6 @@
 // Instantiations and launches of the CTA-per-block FP32 kernels (fsr_coop.cuh).
+#include <algorithm>
+
 #include "fsr_coop.cuh"
 
 namespace fsrk {
@@ -12,7 +14,19 @@ cudaError_t configure_b() {
     if ((e = cudaFuncSetAttribute(coop::fsr_coop_kernel<B, true>, at, bytes)) != cudaSuccess) return e;
     if ((e = cudaFuncSetAttribute(coop::fsr_coop_kernel<B, false>, at, bytes)) != cudaSuccess) return e;
     if ((e = cudaFuncSetAttribute(coop::fsr_coop_reuse_kernel<B, 1>, at, bytes)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(coop::fsr_coop_rows_kernel<B>, at, bytes)) != cudaSuccess) return e;
     return cudaFuncSetAttribute(coop::fsr_coop_reuse_kernel<B, kReuseSegs>, at, bytes);
+}
+
+template <int B>
+cudaError_t launch_rows_b(const coop::RowsArgs& a, int wanted, int sm_count, cudaStream_t stream) {
+    const size_t smem = sizeof(coop::Smem);
+    int grid = 0;
+    cudaError_t e = persistent_grid(coop::fsr_coop_rows_kernel<B>, coop::NW, smem, (long long)wanted * coop::NW,
+                                    sm_count, &grid);
+    if (e != cudaSuccess) return e;
+    coop::fsr_coop_rows_kernel<B><<<grid, coop::T, smem, stream>>>(a);
+    return cudaGetLastError();
 }
 
 template <int B>
@@ -61,6 +75,49 @@ cudaError_t launch_coop(const BatchArgs& a, int B, const ImageArgs* one, cudaStr
         case 16: return launch_b<16>(a, one, stream);
         default: return cudaErrorInvalidValue;
     }
+}
+
+size_t coop_rows_bytes() { return sizeof(unsigned long long) * (coop::kRowRing + 1); }
+
+cudaError_t launch_coop_rows(const MethodArgs& mth, float delta, int n, const ImageArgs* ims, void* ring,
+                             unsigned* status, unsigned long long* empty, int B, int sm_count, cudaStream_t stream) {
+    coop::RowsArgs a = {};
+    a.mth = mth;
+    a.delta = delta;
+    a.lag = (mth.L + B - 1) / B + 1;
+    a.ring = static_cast<unsigned long long*>(ring);
+    a.status = status;
+    a.empty = empty;
+    a.n = n;
+    int order[coop::kRowImages];
+    for (int i = 0; i < n; ++i) order[i] = i;
+    std::stable_sort(order, order + n, [&](int x, int y) { return ims[x].H > ims[y].H; });
+    for (int i = 0; i < n; ++i) {
+        a.im[i] = ims[order[i]];
+        a.nby[i] = (a.im[i].H + B - 1) / B;
+        a.rows += a.nby[i];
+    }
+    const int wanted = (int)coop_rows_parallel(n, ims, mth.L, B);
+    cudaError_t e = cudaMemsetAsync(ring, 0, coop_rows_bytes(), stream);
+    if (e != cudaSuccess) return e;
+    switch (B) {
+        case 2: return launch_rows_b<2>(a, wanted, sm_count, stream);
+        case 4: return launch_rows_b<4>(a, wanted, sm_count, stream);
+        case 8: return launch_rows_b<8>(a, wanted, sm_count, stream);
+        case 16: return launch_rows_b<16>(a, wanted, sm_count, stream);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+long long coop_rows_parallel(int n, const ImageArgs* ims, int L, int B) {
+    const int lag = (L + B - 1) / B + 1;
+    long long p = 0, rows = 0;
+    for (int i = 0; i < n; ++i) {
+        const long long nby = (ims[i].H + B - 1) / B;
+        p += std::min<long long>(nby, ims[i].nbx / lag + 1);
+        rows += nby;
+    }
+    return n <= coop::kRowImages && rows <= 0x7fffffffll ? p : 0x7fffffffll;
 }
 
 cudaError_t launch_coop_reuse(const ReuseLaunch& a, int B, cudaStream_t stream) {

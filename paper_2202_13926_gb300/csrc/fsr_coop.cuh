@@ -453,5 +453,115 @@ __global__ void __launch_bounds__(T) fsr_coop_reuse_kernel(const __grid_constant
     block<B, true, false>(sg.im, by, a.t - a.slope * by, a.mth, sm, a.empty, a.delta);
 }
 
+// Re-use form in one launch: a CTA takes block rows in order and works through
+// a row from left to right; row by of an image runs `lag` = ceil(L / B) + 1
+// blocks behind row by - 1, the same dependency as the wavefront launches
+// (every earlier block of the raster order whose target meets the support is
+// complete), so the results are the same bit for bit.  Against a launch per
+// wavefront it saves the launch and the tables on the chain, and no block
+// waits for the slowest of its wavefront.
+//
+// Rows are claimed in order from a counter, row r of every image before row
+// r + 1 of any (images by falling row count), so the row a CTA waits for is
+// held by a CTA that already runs: the waits end whatever the grid size.
+// Progress of row g is published in ring[g % kRowRing] as (g + 1) << 32 |
+// blocks done (0xffffffff: all); a larger tag in the slot means the row is
+// long done, and a row takes its slot over only from a finished one.
+constexpr int kRowRing = 2048;
+constexpr int kRowImages = 48;
+struct RowsArgs {
+    MethodArgs mth;
+    float delta;
+    int lag, n, rows;            // rows of all images together
+    unsigned long long* ring;    // kRowRing entries, then the row counter: zero at launch
+    unsigned* status;
+    unsigned long long* empty;
+    ImageArgs im[kRowImages];    // by falling number of block rows
+    int nby[kRowImages];
+};
+static_assert(sizeof(RowsArgs) <= 4096, "row launch parameters must fit the 4 KB parameter space");
+
+__device__ __forceinline__ unsigned long long ld_acquire(const unsigned long long* p) {
+    unsigned long long v;
+    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_release(unsigned long long* p, unsigned long long v) {
+    asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+
+// One thread: wait (bounded) until slot shows row g with at least `need`
+// blocks done, or a later row.  The limit is two seconds plus far more than
+// the rows ahead can take (1 us per iteration and block).
+__device__ __forceinline__ bool row_wait(const unsigned long long* slot, unsigned g, unsigned need,
+                                         unsigned long long limit_ns) {
+    unsigned long long t0 = 0, last = 0;
+    for (unsigned it = 0;; ++it) {
+        const unsigned long long v = ld_acquire(slot);
+        const unsigned tag = (unsigned)(v >> 32);
+        if (tag > g + 1u || (tag == g + 1u && (unsigned)v >= need)) return true;
+        __nanosleep(64);
+        if ((it & 63u) == 0u) {
+            unsigned long long t;
+            asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+            if (it == 0u || v != last) t0 = t;   // the clock starts again whenever the row moves on
+            else if (t - t0 > limit_ns) return false;
+            last = v;
+        }
+    }
+}
+
+template <int B>
+__global__ void __launch_bounds__(T) fsr_coop_rows_kernel(const __grid_constant__ RowsArgs a) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ int s_row, s_ok;
+    Smem* sm = reinterpret_cast<Smem*>(smem);
+    tables(a.mth, sm);
+    for (;;) {
+        if (threadIdx.x == 0) s_row = (int)atomicAdd(a.ring + kRowRing, 1ull);
+        __syncthreads();
+        const int g = s_row;
+        if (g >= a.rows) return;
+        // row r of image i: g = (rows r' < r of all images) + i
+        auto before = [&](int r) {
+            int t = 0;
+            for (int i = 0; i < a.n; ++i) t += min(a.nby[i], r);
+            return t;
+        };
+        int lo = 0, hi = a.nby[0] - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (before(mid) <= g) lo = mid;
+            else hi = mid - 1;
+        }
+        const int r = lo, first = before(r), i = g - first;
+        const int prev = r > 0 ? before(r - 1) + i : 0;   // row r - 1 of this image
+        const ImageArgs& im = a.im[i];
+        unsigned long long* slot = a.ring + g % kRowRing;
+        const unsigned long long limit =
+            2000000000ull + 1000ull * (unsigned long long)(im.K + 16) * (unsigned long long)(im.nbx + a.lag);
+        const unsigned long long tag = (unsigned long long)(g + 1) << 32;
+        if (threadIdx.x == 0) {
+            s_ok = g < kRowRing || row_wait(slot, (unsigned)(g - kRowRing), 0xffffffffu, limit);
+            if (s_ok) st_release(slot, tag);
+        }
+        for (int bx = 0; bx < im.nbx; ++bx) {
+            if (threadIdx.x == 0 && r > 0 && s_ok)
+                s_ok = row_wait(a.ring + prev % kRowRing, (unsigned)prev, (unsigned)min(bx + a.lag, im.nbx), limit);
+            __syncthreads();
+            if (!s_ok) {
+                if (threadIdx.x == 0) atomicOr(a.status, kStatusRowWait);
+                return;
+            }
+            block<B, true, false>(im, r, bx, a.mth, sm, a.empty, a.delta);
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                __threadfence();   // the CTA's pixels before the flag
+                st_release(slot, tag | (bx + 1 == im.nbx ? 0xffffffffu : (unsigned)(bx + 1)));
+            }
+        }
+    }
+}
+
 }  // namespace coop
 }  // namespace fsrk

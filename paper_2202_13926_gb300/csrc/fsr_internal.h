@@ -71,5 +71,12 @@ struct fsr_handle {
     cudaEvent_t single_ev[kSingleSlots] = {};
     bool single_used[kSingleSlots] = {};
     unsigned long long single_next = 0;
+    // progress rings of one-launch re-use calls, used in turn (a call waits on
+    // its stream for the last launch that used its slot)
+    static constexpr int kRowSlots = 8;
+    void* d_rows = nullptr;
+    cudaEvent_t row_ev[kRowSlots] = {};
+    bool row_used[kRowSlots] = {};
+    unsigned long long row_next = 0;
     int inject_tile_fault = 0;     // test hook: next tile-copy launch waits for bytes that never come
 };

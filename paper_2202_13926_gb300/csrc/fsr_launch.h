@@ -63,6 +63,19 @@ constexpr int kCoopReusePerSm = 8;
 cudaError_t configure_coop();
 cudaError_t launch_coop(const BatchArgs& a, int B, const ImageArgs* one, cudaStream_t stream);
 cudaError_t launch_coop_reuse(const ReuseLaunch& a, int B, cudaStream_t stream);
+// Re-use form in one launch (fsr_coop_rows_kernel), for calls with at most
+// kCoopRowsPerSm block rows at work per SM (ms, a launch per wavefront / one
+// launch: one 1080p frame, K = 100 53.5 / 45.3; n of them, K = 50: n = 8 (5.1
+// rows per SM) 69.4 / 57.1, 12 (7.7) 88.0 / 78.0, 16 (10.2) 94.3 / 97.4, 24
+// 113 / 142), over `ring`, device memory
+// of coop_rows_bytes() that no other launch uses meanwhile.
+// coop_rows_parallel: the block rows that can be at work at once (the
+// wavefronts' width; 2^31 - 1 for more images than a launch takes).
+constexpr int kCoopRowsPerSm = 8;
+size_t coop_rows_bytes();
+long long coop_rows_parallel(int n, const ImageArgs* ims, int L, int B);
+cudaError_t launch_coop_rows(const MethodArgs& mth, float delta, int n, const ImageArgs* ims, void* ring,
+                             unsigned* status, unsigned long long* empty, int B, int sm_count, cudaStream_t stream);
 
 // Short-lived-CTA form of the FP32 batch kernel (kWarpsFp32 warps, any B),
 // for launches with a.one_round set (the serving loop).
