@@ -566,6 +566,33 @@ __device__ __forceinline__ bool prepare_block(const ImageArgs& a, int y0, int x0
     return true;
 }
 
+// Two floats in one 64-bit register pair.  The state lives in this form, not
+// in float2: carried through the loop as two 32-bit values the pairs come
+// apart and the packed operations are preceded by moves.
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pack2(float x, float y) {
+    f32x2 d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(x), "f"(y));
+    return d;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float& x, float& y) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v));
+}
+__device__ __forceinline__ f32x2 ffma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ f32x2 fmul2(f32x2 a, f32x2 b) {
+    f32x2 d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+// objective() of a pair
+__device__ __forceinline__ f32x2 objective2(f32x2 re, f32x2 im, f32x2 wf) {
+    return fmul2(wf, ffma2(im, im, fmul2(re, re)));
+}
+
 // R = a W + Q for one component (the DC-split representation); the same
 // rounded operations everywhere, so every copy of a value is bit-identical.
 template <typename T>
@@ -1278,7 +1305,9 @@ fsr_batch_kernel(const BatchArgs a) {
         seen = (long long)base;
         bool ok = true;
         for (int sub = 0; sub < take && ok; sub += 32) {
-            unsigned todo = scan_targets<B>(a, seen + sub, min(take - sub, 32), lane);
+            const int n = (int)min((long long)min(take - sub, 32), a.total - (seen + sub));
+            if (n <= 0) break;
+            unsigned todo = scan_targets<B>(a, seen + sub, n, lane);
             while (todo != 0 && ok) {
                 const long long item = seen + sub + (__ffs(todo) - 1);
                 todo &= todo - 1;

@@ -14,12 +14,14 @@
 // so is the selection rule: the results are the same bit for bit.
 //
 // Spectrum layout: warp w holds rows 8w .. 8w + 7, lane (r, g) of it the
-// columns g, g + 4, ..., g + 28 of row 8w + r (r = lane / 4, g = lane % 4).
-// A half-warp then reads 4 rows of 4 consecutive W entries; the row stride of
-// 68 entries of 8 bytes puts them on distinct banks for every shift (u, v).
-// W is stored twice in both directions (64 rows of 64 entries), so the shifted
-// entry W[k-u][l-v] of a thread is one subtraction away from a fixed address:
-// no wrap of either index on the chain from the pick to the W loads.
+// columns g, g + 4, g + 8, g + 12 of row 8w + r (r = lane / 4, g = lane % 4) and
+// those 16 further on, as pairs for packed f32x2 operations.  A stored W row
+// has 48 entries (Re W[c], Re W[c + 16], Im W[c], Im W[c + 16]) of 16 bytes; a
+// quarter-warp reads 2 rows of 4 consecutive entries, which the row stride of
+// 52 entries puts on distinct banks for every shift (u, v).  The rows are
+// stored twice (64 of them), so the shifted entry W[k-u][l-v] of a thread is
+// one subtraction away from a fixed address: no wrap of either index on the
+// chain from the pick to the W loads.
 //
 // Measured (alone on an SM, cycles at 1.98 GHz): one iteration 1,130 with one
 // warp per block, 457 here; of it about 40 the W load, 60 the update,
@@ -38,6 +40,8 @@
 // most of whose time a block that runs alone spends fetching instructions.
 #pragma once
 
+#include <type_traits>
+
 #include "fsr_launch.h"
 
 namespace fsrk {
@@ -46,15 +50,23 @@ namespace coop {
 constexpr int NW = 4;                    // warps per block
 constexpr int T = 32 * NW;               // threads per block
 constexpr int G = 4;                     // lanes per row
-constexpr int NC = S / G;                // components per thread
+constexpr int NP = S / G / 2;             // pairs (l, l + 16) per thread
 constexpr int RPW = S / NW;              // rows per warp
-constexpr int WS = 68;                   // W row stride (float2)
+constexpr int WS = 52;                   // W row stride (16-byte entries)
+constexpr unsigned kDivWS = 65536 / WS + 1;   // off / WS = (off * kDivWS) >> 16 for off < S * WS
+constexpr bool div_ok() {
+    for (unsigned o = 0; o < (unsigned)(S * WS); ++o)
+        if ((o * kDivWS) >> 16 != o / WS) return false;
+    return true;
+}
+static_assert(div_ok(), "division by multiplication");
 constexpr int AS = S + 1;                // row stride of the transform buffers (float2)
 constexpr int H1 = S / 2 + 1;            // w_f quadrant: indices 0 .. S/2
 
 struct Smem {
-    float2 A[S * AS];                    // support (f, w), first transform, spectrum Z
-    float2 W[2 * S * WS];                // exchange buffer of the transforms, then the W rows
+    // the transforms' exchange buffer and A (support (f, w), first transform,
+    // spectrum Z), then the W rows
+    ulonglong2 W[2 * S * WS];
     float4 slot[2][NW];                  // candidates of the warps: maximum, shift offset, coefficient
     float w0[S / 2 * S / 2];             // Eq. (5), one quadrant (symmetric)
     float wf[H1 * H1];                   // Eq. (9), one quadrant (symmetric)
@@ -63,23 +75,34 @@ struct Smem {
     unsigned dmax[NW];
 };
 
+static_assert(2 * sizeof(float2) * S * AS <= sizeof(ulonglong2) * 2 * S * WS, "the transforms fit the W area");
+
 __device__ __forceinline__ int fold(int m) { return m < S / 2 ? m : S - 1 - m; }   // w0: m and S-1-m are alike
 __device__ __forceinline__ int foldf(int k) { return k <= S / 2 ? k : S - k; }      // w_f: k and S-k are alike
 
 // The tables of the CTA: pairs (m, n) with m <= n, both ways round.  Not
-// unrolled: a CTA that runs one block fetches this code cold, and the fetch,
-// not the arithmetic, is its time.
+// unrolled: a CTA that runs one block fetches this code cold, and the fetch is
+// most of its time.  The entries beyond one per thread go to another warp for
+// each table.
 __device__ __forceinline__ void tables(const MethodArgs& mth, Smem* sm) {
+    const int tid = threadIdx.x;
+    constexpr int EF = H1 * (H1 + 1) / 2;          // w_f: 153 pairs, rows r and 16 - r side by side
 #pragma unroll 1
-    for (int i = threadIdx.x; i < H1 * (H1 + 1) / 2; i += T) {
-        // rows r and 16 - r of the triangle side by side: 18 entries
+    for (int p = 0, i = tid; i < EF; i = ++p == 1 ? T + (tid + T - 32) % T : EF) {
         const int r = i / (H1 + 1), c = i % (H1 + 1);
         const bool first = c < H1 - r;
         const int m = first ? r : H1 - 1 - r, n = first ? r + c : c - 1;
         sm->wf[m * H1 + n] = sm->wf[n * H1 + m] = wf_value<float>(mth, m, n);
-        if (n < S / 2) sm->w0[m * (S / 2) + n] = sm->w0[n * (S / 2) + m] = w0_value<float>(mth, m, n);
     }
-    if (threadIdx.x < S) sm->cs[threadIdx.x] = make_float2(float(cos_2pi32(threadIdx.x)), float(sin_2pi32(threadIdx.x)));
+    constexpr int H = S / 2, EW = H * (H + 1) / 2;   // w0: 136 pairs, rows r and 15 - r side by side
+#pragma unroll 1
+    for (int p = 0, i = tid; i < EW; i = ++p == 1 ? T + (tid + T - 64) % T : EW) {
+        const int r = i / (H + 1), c = i % (H + 1);
+        const bool first = c < H - r;
+        const int m = first ? r : H - 1 - r, n = first ? r + c : c - 1;
+        sm->w0[m * H + n] = sm->w0[n * H + m] = w0_value<float>(mth, m, n);
+    }
+    if (tid < S) sm->cs[tid] = make_float2(float(cos_2pi32(tid)), float(sin_2pi32(tid)));
 }
 
 // One butterfly of the FFT, twiddle e^{-j 2 pi tw / 32} = c + j s, with the
@@ -153,6 +176,8 @@ __device__ __forceinline__ void block(const ImageArgs& im, int by, int bx, const
     const long long blk = (long long)by * im.nbx + bx;
     int16_t* seq = im.seq ? im.seq + (size_t)blk * im.K : nullptr;
     const int q2 = ((q & 1) << 1) | (q >> 1);   // the two bits of q reversed
+    float2* X = reinterpret_cast<float2*>(sm->W);
+    float2* A = X + S * AS;
 
     // ---- a1: 8 pixels of column `lane` per thread, and the target pixels ----
     float f[8];
@@ -210,7 +235,7 @@ __device__ __forceinline__ void block(const ImageArgs& im, int by, int bx, const
         const float w0 = sm->w0[fold(m) * (S / 2) + fold(lane)];
         // Eq. (5): w0 on known pixels, delta w0 on re-used ones, 0 elsewhere
         wv[i] = ((kn >> i) & 1u) ? w0 : (((re >> i) & 1u) ? delta * w0 : 0.f);
-        sm->A[m * AS + lane] = make_float2(f[i], wv[i]);
+        A[m * AS + lane] = make_float2(f[i], wv[i]);
     }
     need = __reduce_or_sync(FULL, need | (avail ? 1u : 0u));
     if (lane == 0) sm->flags[q] = need;
@@ -227,9 +252,9 @@ __device__ __forceinline__ void block(const ImageArgs& im, int by, int bx, const
         // ---- a2: sums over the column in row order, then over the columns
         //      (every warp for itself: no barrier); weighted mean ----
         float sw = 0.f, sfw = 0.f;
-#pragma unroll 8
+#pragma unroll
         for (int m = 0; m < S; ++m) {
-            const float2 fw = sm->A[m * AS + lane];
+            const float2 fw = A[m * AS + lane];
             sw = __fadd_rn(sw, fw.y);
             sfw = __fmaf_rn(fw.y, fw.x, sfw);
         }
@@ -264,40 +289,59 @@ __device__ __forceinline__ void block(const ImageArgs& im, int by, int bx, const
 #pragma unroll 1
         for (int pass = 0; pass < 2; ++pass) {
             float2 e[2][4];
-            fft32_split(x, e, sm->W, sm->cs, q, lane);
+            fft32_split(x, e, X, sm->cs, q, lane);
             // first transform out by rows k, then back in by columns; the second stays transposed
             const int sk = pass == 0 ? AS : 1, sl = pass == 0 ? 1 : AS;
 #pragma unroll
             for (int tt = 0; tt < 2; ++tt)
 #pragma unroll
-                for (int p = 0; p < 4; ++p) sm->A[(2 * q + tt + 8 * p) * sk + lane * sl] = e[tt][p];
+                for (int p = 0; p < 4; ++p) A[(2 * q + tt + 8 * p) * sk + lane * sl] = e[tt][p];
             __syncthreads();
             if (pass == 0) {
 #pragma unroll
-                for (int i = 0; i < 8; ++i) x[i] = sm->A[lane * AS + in_index(q2, i)];
+                for (int i = 0; i < 8; ++i) x[i] = A[lane * AS + in_index(q2, i)];
             }
         }
 
         // ---- Q and W of this thread's components ----
         const int k = RPW * q + lane / G, g = lane % G;
-        float zr[NC], zi[NC], wf[NC], o[NC];
-        float2 wu[NC];   // the unshifted W row (DC phase)
+        f32x2 zr[NP], zi[NP], wf[NP], wur[NP], wui[NP];   // wu: the unshifted W row (DC phase)
 #pragma unroll
-        for (int j = 0; j < NC; ++j) {
-            const int l = g + G * j;
-            const float2 a = sm->A[k * AS + l], c = sm->A[((S - k) & (S - 1)) * AS + ((S - l) & (S - 1))];
-            wu[j] = make_float2((a.y + c.y) * inv2alpha, (c.x - a.x) * inv2alpha);
-            zr[j] = (a.x + c.x) * 0.5f;
-            zi[j] = (a.y - c.y) * 0.5f;
-            wf[j] = sm->wf[foldf(k) * H1 + foldf(l)];
+        for (int j = 0; j < NP; ++j) {
+            float qr[2], qi[2], wr[2], wi[2], f2[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int l = g + G * j + S / 2 * h;
+                const float2 a = A[k * AS + l], c = A[((S - k) & (S - 1)) * AS + ((S - l) & (S - 1))];
+                wr[h] = (a.y + c.y) * inv2alpha;
+                wi[h] = (c.x - a.x) * inv2alpha;
+                qr[h] = (a.x + c.x) * 0.5f;
+                qi[h] = (a.y - c.y) * 0.5f;
+                f2[h] = sm->wf[foldf(k) * H1 + foldf(l)];
+            }
+            zr[j] = pack2(qr[0], qr[1]);
+            zi[j] = pack2(qi[0], qi[1]);
+            wf[j] = pack2(f2[0], f2[1]);
+            wur[j] = pack2(wr[0], wr[1]);
+            wui[j] = pack2(wi[0], wi[1]);
         }
+        __syncthreads();   // Z is read no more: the W rows go there
 #pragma unroll
-        for (int j = 0; j < NC; ++j) {
-            float2* w = sm->W + k * WS + g + G * j;
-            w[0] = w[S] = w[S * WS] = w[S * WS + S] = wu[j];
+        for (int j = 0; j < NP; ++j) {
+            // entries l, l + 16 (the halves change places) and l + 32, in rows k and k + 32
+            float r0, r1, i0, i1;
+            unpack2(wur[j], r0, r1);
+            unpack2(wui[j], i0, i1);
+            const ulonglong2 e = make_ulonglong2(wur[j], wui[j]);
+            const ulonglong2 x = make_ulonglong2(pack2(r1, r0), pack2(i1, i0));
+            ulonglong2* w = sm->W + k * WS + g + G * j;
+            w[0] = w[S] = w[S * WS] = w[S * WS + S] = e;
+            w[S / 2] = w[S * WS + S / 2] = x;
         }
         __syncthreads();
-        const float cg = mth.gamma * (1.f / sm->W[0].x);
+        float w00, w16;
+        unpack2(sm->W[0].x, w00, w16);
+        const float cg = mth.gamma * (1.f / w00);
         int pm[PT], pn[PT];
 #pragma unroll
         for (int p = 0; p < PT; ++p) {
@@ -305,12 +349,11 @@ __device__ __forceinline__ void block(const ImageArgs& im, int by, int bx, const
             pn[p] = L + (tid + T * p) % B;
         }
         // W[k-u][l-v] lies u rows and v entries before this one
-        const float2* wbase = sm->W + (k + S) * WS + g + S;
-        const unsigned idx0 = (unsigned)(k * S + g);
-        int16_t* seq0 = tid == 0 ? seq : nullptr;
+        const ulonglong2* wbase = sm->W + (k + S) * WS + g + S;
+        const unsigned off0 = (unsigned)(k * WS + g);
         float cr = 0.f, ci = 0.f;
         unsigned off;   // u * WS + v
-        float m;        // this thread's maximum
+        float olo[NP] = {}, ohi[NP] = {};   // objectives of the pairs' halves
         float2 csn[PT];
 #pragma unroll
         for (int p = 0; p < PT; ++p) csn[p] = make_float2(0.f, 0.f);
@@ -320,31 +363,42 @@ __device__ __forceinline__ void block(const ImageArgs& im, int by, int bx, const
             for (int p = 0; p < PT; ++p) gacc[p] = fma_rn(cr, csn[p].x, fma_rn(-ci, csn[p].y, gacc[p]));
         };
 
-        // a5, a6 for the objectives o[] of the values (vr, vi): the warp's
+        // a5, a6 for the objectives of the values (vr, vi): the warp's
         // maximum (objectives are >= +0: their bits order like the values)
         // and its lowest index, then the four warps' candidates.  What a
-        // thread would publish is formed while the reductions run.
-        auto pick = [&](int nu, const float (&vr)[NC], const float (&vi)[NC]) {
+        // thread may publish is formed while the reductions run: its lowest
+        // component holding its own maximum, by halving.
+        auto pick = [&](int nu, const f32x2 (&vr)[NP], const f32x2 (&vi)[NP]) {
+            const float mlo = fmaxf(max3(olo[0], olo[1], olo[2]), olo[3]);
+            const float mhi = fmaxf(max3(ohi[0], ohi[1], ohi[2]), ohi[3]);
+            const float m = fmaxf(mlo, mhi);
             const unsigned mb = __float_as_uint(m);
             const unsigned Mw = __reduce_max_sync(FULL, mb);
             target();   // of the previous pick
-            unsigned jj[NC];
+            const bool h1 = __float_as_uint(mlo) == mb;   // columns < 16
+            float o1[3], r1[NP], i1[NP];
 #pragma unroll
-            for (int j = 0; j < NC; ++j) jj[j] = __float_as_uint(o[j]) == mb ? (unsigned)j : (unsigned)(NC - 1);
-            const unsigned bj = min(min(min(jj[0], jj[1]), min(jj[2], jj[3])), min(min(jj[4], jj[5]), min(jj[6], jj[7])));
-            const unsigned bidx = idx0 + G * bj;
-            const unsigned lo = __reduce_min_sync(FULL, mb == Mw ? bidx : (unsigned)(S * S));
-            float br = vr[NC - 1], bi = vi[NC - 1];
-#pragma unroll
-            for (int j = NC - 2; j >= 0; --j) {
-                const bool h = __float_as_uint(o[j]) == mb;
-                br = h ? vr[j] : br;
-                bi = h ? vi[j] : bi;
+            for (int j = 0; j < NP; ++j) {
+                float r0, rx, i0, ix;
+                unpack2(vr[j], r0, rx);
+                unpack2(vi[j], i0, ix);
+                if (j < 3) o1[j] = h1 ? olo[j] : ohi[j];
+                r1[j] = h1 ? r0 : rx;
+                i1[j] = h1 ? i0 : ix;
             }
-            // c = gamma p (Eq. 10); index u * S + v as the offset u * WS + v
-            const float4 mine = make_float4(m, __uint_as_float((bidx >> 5) * WS + (bidx & (S - 1))), br * cg, bi * cg);
+            const bool h2 = __float_as_uint(fmaxf(o1[0], o1[1])) == mb;   // of those the first two
+            const float o2 = h2 ? o1[0] : o1[2];
+            const float r20 = h2 ? r1[0] : r1[2], r21 = h2 ? r1[1] : r1[3];
+            const float i20 = h2 ? i1[0] : i1[2], i21 = h2 ? i1[1] : i1[3];
+            const bool h3 = __float_as_uint(o2) == mb;
+            const float br = h3 ? r20 : r21, bi = h3 ? i20 : i21;
+            // index u * S + v as the offset u * WS + v: the same order
+            const unsigned boff = off0 + (h1 ? 0u : S / 2) + (h2 ? 0u : 2u * G) + (h3 ? 0u : (unsigned)G);
+            const unsigned lo = __reduce_min_sync(FULL, mb == Mw ? boff : 0xffffffffu);
+            // c = gamma p (Eq. 10)
+            const float4 mine = make_float4(m, __uint_as_float(boff), br * cg, bi * cg);
             float4* sl = sm->slot[nu & 1];
-            if (mb == Mw && bidx == lo) sl[q] = mine;
+            if (mb == Mw && boff == lo) sl[q] = mine;
             __syncthreads();   // one barrier per iteration: the slots alternate
             // rows ascend with the warp, so the first maximum has the lowest index
             float4 c0 = sl[0], c2 = sl[2];
@@ -355,45 +409,70 @@ __device__ __forceinline__ void block(const ImageArgs& im, int by, int bx, const
             off = __float_as_uint(c0.y);
             cr = c0.z;
             ci = c0.w;
-            const int u = (int)(off / WS), v = (int)(off % WS);
-            if (seq0 != nullptr) seq0[nu] = (int16_t)(u * S + v);
+        };
+        // the recorded index, and the target pixels' phases of the pick (used
+        // by target() in the next one)
+        // (in every thread: a branch to the warps that have target pixels costs
+        // 50 cycles of the iteration)
+        auto note = [&](int nu, auto rec) {
+            const int u = (int)((off * kDivWS) >> 16), v = (int)(off - (unsigned)u * WS);
+            if constexpr (rec.value) {
+                if (tid == 0) seq[nu] = (int16_t)(u * S + v);
+            }
 #pragma unroll
             for (int p = 0; p < PT; ++p) csn[p] = sm->cs[(u * pm[p] + v * pn[p]) & (S - 1)];
         };
-        auto max_all = [&]() { m = max3(max3(o[0], o[1], o[2]), max3(o[3], o[4], o[5]), fmaxf(o[6], o[7])); };
 
-        // ---- a4-a8: the DC phase, R = a W + Q, then the plain loop ----
-        int nu = 0;
-        {
-            float ar = mu, ai = 0.f;
-            for (;;) {
-                float rr[NC], ri[NC];
+        // ---- a4-a8: the DC phase, R = a W + Q, then the plain loop; rec: the
+        //      selected indices are recorded ----
+        auto iterate = [&](auto rec) {
+            int nu = 0;
+            {
+                float ar = mu, ai = 0.f;
+                for (;;) {
+                    const f32x2 ar2 = pack2(ar, ar), ai2 = pack2(ai, ai), nai2 = pack2(-ai, -ai);
+                    f32x2 rr[NP], ri[NP];
 #pragma unroll
-                for (int j = 0; j < NC; ++j) {
-                    split_value(ar, ai, wu[j].x, wu[j].y, zr[j], zi[j], rr[j], ri[j]);
-                    o[j] = objective<float>(rr[j], ri[j], wf[j]);
+                    for (int j = 0; j < NP; ++j) {
+                        rr[j] = ffma2(ar2, wur[j], ffma2(nai2, wui[j], zr[j]));
+                        ri[j] = ffma2(ar2, wui[j], ffma2(ai2, wur[j], zi[j]));
+                        unpack2(objective2(rr[j], ri[j], wf[j]), olo[j], ohi[j]);
+                    }
+                    pick(nu, rr, ri);
+                    if (nu + 1 == K || off != 0) {
+#pragma unroll
+                        for (int j = 0; j < NP; ++j) {   // fold a W into Q
+                            zr[j] = rr[j];
+                            zi[j] = ri[j];
+                        }
+                        break;
+                    }
+                    note(nu++, rec);
+                    ar -= cr;
+                    ai -= ci;
                 }
-                max_all();
-                pick(nu, rr, ri);
-                if (++nu == K || off != 0) break;
-                ar -= cr;
-                ai -= ci;
             }
+            for (;;) {   // the pick of iteration nu is not applied yet
+                if (nu + 1 == K) break;
+                const ulonglong2* row = wbase - off;   // a7 (Eq. 12) and the next objective
+                ulonglong2 w[NP];
 #pragma unroll
-            for (int j = 0; j < NC; ++j) split_value(ar, ai, wu[j].x, wu[j].y, zr[j], zi[j], zr[j], zi[j]);
-        }
-        while (nu < K) {
-            const float2* row = wbase - off;   // a7 (Eq. 12) and the next objective
+                for (int j = 0; j < NP; ++j) w[j] = row[G * j];
+                note(nu++, rec);   // while the loads are under way
+                const f32x2 ncr2 = pack2(-cr, -cr), ci2 = pack2(ci, ci), nci2 = pack2(-ci, -ci);
 #pragma unroll
-            for (int j = 0; j < NC; ++j) {
-                const float2 w = row[G * j];
-                residual_update(zr[j], zi[j], w.x, w.y, cr, ci);
-                o[j] = objective<float>(zr[j], zi[j], wf[j]);
+                for (int j = 0; j < NP; ++j) {
+                    zr[j] = ffma2(ncr2, w[j].x, ffma2(ci2, w[j].y, zr[j]));
+                    zi[j] = ffma2(ncr2, w[j].y, ffma2(nci2, w[j].x, zi[j]));
+                    unpack2(objective2(zr[j], zi[j], wf[j]), olo[j], ohi[j]);
+                }
+                pick(nu, zr, zi);
             }
-            max_all();
-            pick(nu++, zr, zi);
-        }
-        target();
+            note(nu, rec);
+            target();
+        };
+        if (seq != nullptr) iterate(std::true_type{});
+        else iterate(std::false_type{});
     }
 
     // ---- a9 ----
@@ -536,7 +615,7 @@ __global__ void __launch_bounds__(T) fsr_coop_rows_kernel(const __grid_constant_
         }
         const int r = lo, first = before(r), i = g - first;
         const int prev = r > 0 ? before(r - 1) + i : 0;   // row r - 1 of this image
-        const ImageArgs& im = a.im[i];
+        const ImageArgs im = a.im[i];
         unsigned long long* slot = a.ring + g % kRowRing;
         const unsigned long long limit =
             2000000000ull + 1000ull * (unsigned long long)(im.K + 16) * (unsigned long long)(im.nbx + a.lag);
@@ -545,9 +624,12 @@ __global__ void __launch_bounds__(T) fsr_coop_rows_kernel(const __grid_constant_
             s_ok = g < kRowRing || row_wait(slot, (unsigned)(g - kRowRing), 0xffffffffu, limit);
             if (s_ok) st_release(slot, tag);
         }
+        __syncthreads();
         for (int bx = 0; bx < im.nbx; ++bx) {
-            if (threadIdx.x == 0 && r > 0 && s_ok)
-                s_ok = row_wait(a.ring + prev % kRowRing, (unsigned)prev, (unsigned)min(bx + a.lag, im.nbx), limit);
+            // the row above, while thread 0 publishes the last block
+            if (threadIdx.x == T - 1 && r > 0 && s_ok &&
+                !row_wait(a.ring + prev % kRowRing, (unsigned)prev, (unsigned)min(bx + a.lag, im.nbx), limit))
+                s_ok = 0;
             __syncthreads();
             if (!s_ok) {
                 if (threadIdx.x == 0) atomicOr(a.status, kStatusRowWait);
@@ -555,10 +637,8 @@ __global__ void __launch_bounds__(T) fsr_coop_rows_kernel(const __grid_constant_
             }
             block<B, true, false>(im, r, bx, a.mth, sm, a.empty, a.delta);
             __syncthreads();
-            if (threadIdx.x == 0) {
-                __threadfence();   // the CTA's pixels before the flag
-                st_release(slot, tag | (bx + 1 == im.nbx ? 0xffffffffu : (unsigned)(bx + 1)));
-            }
+            // (release at the end of a barrier: the CTA's pixels come before it)
+            if (threadIdx.x == 0) st_release(slot, tag | (bx + 1 == im.nbx ? 0xffffffffu : (unsigned)(bx + 1)));
         }
     }
 }

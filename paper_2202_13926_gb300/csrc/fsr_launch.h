@@ -51,14 +51,15 @@ cudaError_t launch_batch_small(const BatchArgs& a, int S, int B, int fp64, int c
 // blocks.  A block that has an SM (nearly) to itself is done in half the time
 // of the one-warp kernel; with more of them the four warps of a block cost
 // more issue slots than its one warp does.  The lines, measured:
-//   independent blocks, K = 100, us per call, one-warp / CTA-per-block kernel:
-//   0.4 blocks per SM 75 / 31, 2.2 75 / 46, 3.8 74 / 58, 6.7 75 / 104;
+//   independent blocks, us per call, one-warp / CTA-per-block kernel: 0.4
+//   blocks per SM K = 100 75 / 29, 2.2 74 / 41, 3.8 73 / 49, 4.4 74 / 68, 5.9
+//   74 / 74 (K = 25 35 / 33), 6.7 74 / 82 (K = 25 35 / 35);
 //   re-use form, K = 50, ms for n 1080p frames together with the line at 0, 4,
 //   6, 8, 10, 16 blocks per SM: n = 8 98, 82, 68, 68, 68, 69; n = 16 103, 97,
 //   95, 94, 96, 113; n = 24 120, 115, 114, 113, 115, 160.
 // `one`: a single image as kernel parameters (no work table), or nullptr for
 // the table of a.
-constexpr int kCoopBlocksPerSm = 4;
+constexpr int kCoopBlocksPerSm = 6;
 constexpr int kCoopReusePerSm = 8;
 cudaError_t configure_coop();
 cudaError_t launch_coop(const BatchArgs& a, int B, const ImageArgs* one, cudaStream_t stream);

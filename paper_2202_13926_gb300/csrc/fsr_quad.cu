@@ -109,33 +109,6 @@ __device__ __forceinline__ void fftn(float (&re)[N], float (&im)[N]) {
     }
 }
 
-// Two floats in one 64-bit register pair.  The state lives in this form, not
-// in float2: carried through the loop as two 32-bit values the pairs come
-// apart and the packed operations are preceded by moves.
-using f32x2 = unsigned long long;
-__device__ __forceinline__ f32x2 pack2(float x, float y) {
-    f32x2 d;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(x), "f"(y));
-    return d;
-}
-__device__ __forceinline__ void unpack2(f32x2 v, float& x, float& y) {
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v));
-}
-__device__ __forceinline__ f32x2 ffma2(f32x2 a, f32x2 b, f32x2 c) {
-    f32x2 d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ f32x2 fmul2(f32x2 a, f32x2 b) {
-    f32x2 d;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-// objective() of a pair
-__device__ __forceinline__ f32x2 objective2(f32x2 re, f32x2 im, f32x2 wf) {
-    return fmul2(wf, ffma2(im, im, fmul2(re, re)));
-}
-
 // reductions inside a group of SZ lanes
 __device__ __forceinline__ unsigned group_umax(unsigned v) {
 #pragma unroll
