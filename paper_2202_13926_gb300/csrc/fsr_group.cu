@@ -351,7 +351,14 @@ __device__ __forceinline__ void group_block(const ImageArgs& im, long long blk, 
             u = ub ? __ffs(ub) - 1 : 0;
         }
         __syncwarp();   // the previous pick's reads of the published row are done
-        if (run && t == u) {
+        if constexpr (SZ == 16) {
+            const uint32_t ad = smem_addr(rowbuf);
+#pragma unroll
+            for (int c = 0; c < SZ; c += 8)
+                st_shared_64(ad + 8 * c, run && t == u, zr[c], zi[c], zr[c + 1], zi[c + 1], zr[c + 2], zi[c + 2], zr[c + 3],
+                             zi[c + 3], zr[c + 4], zi[c + 4], zr[c + 5], zi[c + 5], zr[c + 6], zi[c + 6], zr[c + 7],
+                             zi[c + 7]);
+        } else if (run && t == u) {
             float4* pub = reinterpret_cast<float4*>(rowbuf);
 #pragma unroll
             for (int i = 0; i < SZ / 2; ++i) pub[i] = make_float4(zr[2 * i], zi[2 * i], zr[2 * i + 1], zi[2 * i + 1]);
@@ -380,7 +387,7 @@ __device__ __forceinline__ void group_block(const ImageArgs& im, long long blk, 
             }
         }
         // a7 (Eq. 12) and the objective of the next iteration (this group only)
-        if (run && nu + 1 < Kr) {
+        if (all || (run && nu + 1 < Kr)) {   // (a last update nobody reads costs less than a branch in every iteration)
             if (dc && split && (u | v) == 0) {
                 ar -= cr;
                 ai -= ci;

@@ -717,7 +717,16 @@ __device__ __forceinline__ void block(const ImageArgs& im, long long blk, int L,
                     // first lane that meets Mx has the lowest linear index.
                     const int ul = __ffs(cands) - 1;
                     __syncwarp();   // the previous pick's reads of pub are done
-                    if (lane == ul) {
+                    if constexpr (sizeof(T) == 4) {
+                        static_assert(P == 18, "S = 24");
+                        const uint32_t ad = smem_addr(pub);
+#pragma unroll
+                        for (int c = 0; c < 16; c += 8)
+                            st_shared_64(ad + 8 * c, lane == ul, zr[c], zi[c], zr[c + 1], zi[c + 1], zr[c + 2],
+                                         zi[c + 2], zr[c + 3], zi[c + 3], zr[c + 4], zi[c + 4], zr[c + 5], zi[c + 5],
+                                         zr[c + 6], zi[c + 6], zr[c + 7], zi[c + 7]);
+                        if (lane == ul) *reinterpret_cast<float4*>(pub + 16) = make_float4(zr[16], zi[16], zr[17], zi[17]);
+                    } else if (lane == ul) {
 #pragma unroll
                         for (int p = 0; p < P; ++p) {
                             T2 e;
@@ -762,6 +771,27 @@ __device__ __forceinline__ void block(const ImageArgs& im, long long blk, int L,
     }
 }
 
+// The target of block blk when all its pixels are known: copied (see
+// scan_targets), a pixel per lane.
+template <int B>
+__device__ __forceinline__ bool copy_if_known(const ImageArgs& im, long long blk, int lane) {
+    constexpr int PT = TargetPix<B>::P;
+    const int by = (int)(blk / im.nbx), bx = (int)(blk - (long long)by * im.nbx);
+    bool unknown = false;
+#pragma unroll
+    for (int q = 0; q < PT; ++q) {
+        const int i = lane + 32 * q, ty = by * B + i / B, tx = bx * B + i % B;
+        if (i < B * B && ty < im.H && tx < im.W) unknown |= __ldg(im.mask + (size_t)ty * im.pitch + tx) == 0;
+    }
+    if (__any_sync(FULL, unknown)) return false;
+#pragma unroll
+    for (int q = 0; q < PT; ++q) {
+        const int i = lane + 32 * q, ty = by * B + i / B, tx = bx * B + i % B;
+        if (i < B * B && ty < im.H && tx < im.W) im.out[(size_t)ty * im.pitch + tx] = __ldg(im.img + (size_t)ty * im.pitch + tx);
+    }
+    return true;
+}
+
 template <typename T, int SZ, int B>
 __device__ __forceinline__ void run(const BatchArgs& a) {
     using Lay = Layout<T, SZ>;
@@ -792,7 +822,7 @@ __device__ __forceinline__ void run(const BatchArgs& a) {
                 else hi = mid - 1;
             }
             const ImageArgs im = a.images[lo];
-            if (scan_targets<B>(a, item, 1, lane) == 0u) continue;   // all targets known: copied
+            if (im.seq == nullptr && copy_if_known<B>(im, item - __ldg(a.first + lo), lane)) continue;
             block<T, SZ, B>(im, item - __ldg(a.first + lo), a.mth.L, gamma, sw0, swf, stw, stt, area, a.empty,
                             lane);
         }
