@@ -232,7 +232,7 @@ int enqueue_single_fp32(fsr_handle* h, const float* img, const uint8_t* mask, in
         a.mth = method_args(p);
         a.empty = h->d_empty;
         const fsrk::ImageArgs im = image_args(img, mask, out, p->seq_out, height, width, pitch, p->iters, p->block);
-        if ((e = fsrk::launch_coop(a, p->block, &im, stream)) != cudaSuccess)
+        if ((e = fsrk::launch_coop(a, p->block, &im, h->sm_count, stream)) != cudaSuccess)
             return fail(h, FSR_ERR_CUDA, "kernel launch failed: %s", cudaGetErrorString(e));
         return ok(h);
     }

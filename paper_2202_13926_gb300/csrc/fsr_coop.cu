@@ -9,10 +9,10 @@ namespace {
 template <int B>
 cudaError_t configure_b() {
     cudaError_t e;
-    const int bytes = (int)sizeof(coop::Smem);
+    const int bytes = (int)sizeof(coop::Smem<4>);
     const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    if ((e = cudaFuncSetAttribute(coop::fsr_coop_kernel<B, true>, at, bytes)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(coop::fsr_coop_kernel<B, false>, at, bytes)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(coop::fsr_coop_kernel<B, 4, true>, at, bytes)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(coop::fsr_coop_kernel<B, 4, false>, at, bytes)) != cudaSuccess) return e;
     if ((e = cudaFuncSetAttribute(coop::fsr_coop_reuse_kernel<B, 1>, at, bytes)) != cudaSuccess) return e;
     if ((e = cudaFuncSetAttribute(coop::fsr_coop_rows_kernel<B>, at, bytes)) != cudaSuccess) return e;
     return cudaFuncSetAttribute(coop::fsr_coop_reuse_kernel<B, kReuseSegs>, at, bytes);
@@ -20,20 +20,20 @@ cudaError_t configure_b() {
 
 template <int B>
 cudaError_t launch_rows_b(const coop::RowsArgs& a, int wanted, int sm_count, cudaStream_t stream) {
-    const size_t smem = sizeof(coop::Smem);
+    const size_t smem = sizeof(coop::Smem<4>);
     int grid = 0;
-    cudaError_t e = persistent_grid(coop::fsr_coop_rows_kernel<B>, coop::NW, smem, (long long)wanted * coop::NW,
+    cudaError_t e = persistent_grid(coop::fsr_coop_rows_kernel<B>, 4, smem, (long long)wanted * 4,
                                     sm_count, &grid);
     if (e != cudaSuccess) return e;
-    coop::fsr_coop_rows_kernel<B><<<grid, coop::T, smem, stream>>>(a);
+    coop::fsr_coop_rows_kernel<B><<<grid, coop::Cfg<4>::T, smem, stream>>>(a);
     return cudaGetLastError();
 }
 
 template <int B>
 cudaError_t launch_b(const BatchArgs& a, const ImageArgs* one, cudaStream_t stream) {
-    const size_t smem = sizeof(coop::Smem);
-    if (one) coop::fsr_coop_kernel<B, true><<<(unsigned)a.total, coop::T, smem, stream>>>(a, *one);
-    else coop::fsr_coop_kernel<B, false><<<(unsigned)a.total, coop::T, smem, stream>>>(a, ImageArgs());
+    const size_t smem = sizeof(coop::Smem<4>);
+    if (one) coop::fsr_coop_kernel<B, 4, true><<<(unsigned)a.total, coop::Cfg<4>::T, smem, stream>>>(a, *one);
+    else coop::fsr_coop_kernel<B, 4, false><<<(unsigned)a.total, coop::Cfg<4>::T, smem, stream>>>(a, ImageArgs());
     return cudaGetLastError();
 }
 
@@ -41,8 +41,8 @@ template <int B, int NSEG>
 cudaError_t launch_reuse_n(const ReuseLaunchN<NSEG>& a, cudaStream_t stream) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)a.total);
-    cfg.blockDim = dim3(coop::T);
-    cfg.dynamicSmemBytes = sizeof(coop::Smem);
+    cfg.blockDim = dim3(coop::Cfg<4>::T);
+    cfg.dynamicSmemBytes = sizeof(coop::Smem<4>);
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -60,14 +60,16 @@ cudaError_t launch_reuse_b(const ReuseLaunch& a, cudaStream_t stream) {
 }  // namespace
 
 cudaError_t configure_coop() {
-    cudaError_t e;
+    cudaError_t e = configure_coop2();
+    if (e != cudaSuccess) return e;
     if ((e = configure_b<2>()) != cudaSuccess) return e;
     if ((e = configure_b<4>()) != cudaSuccess) return e;
     if ((e = configure_b<8>()) != cudaSuccess) return e;
     return configure_b<16>();
 }
 
-cudaError_t launch_coop(const BatchArgs& a, int B, const ImageArgs* one, cudaStream_t stream) {
+cudaError_t launch_coop(const BatchArgs& a, int B, const ImageArgs* one, int sm_count, cudaStream_t stream) {
+    if (a.total > (long long)kCoop4BlocksPerSm * sm_count) return launch_coop2(a, B, one, stream);
     switch (B) {
         case 2: return launch_b<2>(a, one, stream);
         case 4: return launch_b<4>(a, one, stream);

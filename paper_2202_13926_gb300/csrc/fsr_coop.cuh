@@ -1,38 +1,42 @@
-// FP32 FSR at S = 32 with a CTA of four warps on one support block, for calls
-// with few blocks in flight: the 32 x 32 spectrum is spread over 128 threads,
-// 8 components each.
+// FP32 FSR at S = 32 with a CTA of four or two warps on one support block, for
+// calls with few blocks in flight: the 32 x 32 spectrum is spread over 128
+// threads, 8 components each (or 64 threads, 16 each).
 //
 // What bounds it: the K iterations of a block are a serial chain (the argmax
 // of Eq. (8) needs the residual of Eq. (12), which needs the last argmax), so
 // such a call pays the latency of one iteration K times.  One warp per block
 // (fsr_block.cuh) walks 32 components per lane in every iteration; here the
 // update and the objective of a thread are 8 independent components, and one
-// CTA barrier per iteration joins the four warps' maxima.
+// CTA barrier per iteration joins the warps' maxima.  Four warps have the
+// shortest chain, two need fewer issue slots per block: which one a launch
+// takes goes by its blocks per SM (fsr_launch.h).
 //
 // The arithmetic of every component, of both transforms, of the objective and
 // of the target pixels is that of fsr_block.cuh operation by operation, and
 // so is the selection rule: the results are the same bit for bit.
 //
-// Spectrum layout: warp w holds rows 8w .. 8w + 7, lane (r, g) of it the
-// columns g, g + 4, g + 8, g + 12 of row 8w + r (r = lane / 4, g = lane % 4) and
-// those 16 further on, as pairs for packed f32x2 operations.  A stored W row
-// has 48 entries (Re W[c], Re W[c + 16], Im W[c], Im W[c + 16]) of 16 bytes; a
-// quarter-warp reads 2 rows of 4 consecutive entries, which the row stride of
+// Spectrum layout (four warps): warp w holds rows 8w .. 8w + 7, lane (r, g) of
+// it the columns g, g + 4, g + 8, g + 12 of row 8w + r (r = lane / 4, g = lane %
+// 4) and those 16 further on, as pairs for packed f32x2 operations.  A stored W
+// row has 48 entries (Re W[c], Re W[c + 16], Im W[c], Im W[c + 16]) of 16 bytes;
+// a quarter-warp reads 2 rows of 4 consecutive entries, which the row stride of
 // 52 entries puts on distinct banks for every shift (u, v).  The rows are
 // stored twice (64 of them), so the shifted entry W[k-u][l-v] of a thread is
 // one subtraction away from a fixed address: no wrap of either index on the
 // chain from the pick to the W loads.
 //
-// Measured (alone on an SM, cycles at 1.98 GHz): one iteration 1,130 with one
-// warp per block, 457 here; of it about 40 the W load, 60 the update,
-// objective and maximum, 70 two warp reductions, 90 the barrier and the
-// candidates through shared memory.  What a thread may publish, and the
-// target pixels of the previous pick, are computed while the reductions run.
-// 8 and 16 warps per block: 480-600 (more candidates to read and more warps
-// at the barrier), at more issue slots.
+// Measured (a block alone on an SM, cycles at 1.98 GHz): one iteration takes
+// 1,130 with one warp per block, 385 with four: about 40 the W load, 50 the
+// update, objective and maximum, 65 two warp reductions, 90 the barrier and the
+// candidates through shared memory; the rest is issue.  What a thread may
+// publish, and the target pixels of the previous pick, are computed while the
+// reductions and loads run.  A branch in this chain costs 40 to 60 cycles even
+// when every thread goes the same way, so the loop has none.  Scalar
+// components instead of pairs: 457; 8 and 16 warps per block: 480-600.
 //
-// Transforms: the radix-2 decimation-in-time FFT of length 32 splits over the
-// warps.  Warp q takes the inputs of rows (columns) = brev2(q) mod 4, does
+// Transforms (four warps): the radix-2 decimation-in-time FFT of length 32
+// splits over the warps.  Warp q takes the inputs of rows (columns) = brev2(q)
+// mod 4, does
 // the three stages inside its 8 points in registers, and after one exchange
 // through shared memory the last two stages of the points t, t + 8, t + 16,
 // t + 24 for t = 2q, 2q + 1.  A thread so runs about 200 instructions per
@@ -47,35 +51,46 @@
 namespace fsrk {
 namespace coop {
 
-constexpr int NW = 4;                    // warps per block
-constexpr int T = 32 * NW;               // threads per block
-constexpr int G = 4;                     // lanes per row
-constexpr int NP = S / G / 2;             // pairs (l, l + 16) per thread
-constexpr int RPW = S / NW;              // rows per warp
-constexpr int WS = 52;                   // W row stride (16-byte entries)
-constexpr unsigned kDivWS = 65536 / WS + 1;   // off / WS = (off * kDivWS) >> 16 for off < S * WS
-constexpr bool div_ok() {
-    for (unsigned o = 0; o < (unsigned)(S * WS); ++o)
-        if ((o * kDivWS) >> 16 != o / WS) return false;
-    return true;
-}
-static_assert(div_ok(), "division by multiplication");
+// Shape of the kernel with N warps per block.
+template <int N>
+struct Cfg {
+    static_assert(N == 4 || N == 2, "4 or 2 warps per block");
+    static constexpr int T = 32 * N;             // threads per block
+    static constexpr int G = N;                  // lanes per row
+    static constexpr int NP = S / G / 2;         // pairs (l, l + 16) per thread
+    static constexpr int RPW = S / N;            // rows per warp
+    static constexpr int WS = N == 4 ? 52 : 50;  // W row stride (16-byte entries)
+    // 4 warps: rows stored twice, the shifted row is one subtraction away; 2
+    // warps: once, so that 8 CTAs share an SM (28 KB, 128 registers)
+    static constexpr bool TWICE = N == 4;
+    static constexpr int MIN_CTAS = N == 4 ? 1 : 8;
+    static constexpr int PTS = S / N;            // points of a transform per thread
+    static constexpr int TT = PTS / N;           // groups of N points in its last stages
+    static constexpr unsigned DIV = 65536 / WS + 1;   // off / WS = (off * DIV) >> 16 for off < S * WS
+    static constexpr bool div_ok() {
+        for (unsigned o = 0; o < (unsigned)(S * WS); ++o)
+            if ((o * DIV) >> 16 != o / WS) return false;
+        return true;
+    }
+};
+static_assert(Cfg<4>::div_ok() && Cfg<2>::div_ok(), "division by multiplication");
 constexpr int AS = S + 1;                // row stride of the transform buffers (float2)
 constexpr int H1 = S / 2 + 1;            // w_f quadrant: indices 0 .. S/2
 
+template <int N>
 struct Smem {
     // the transforms' exchange buffer and A (support (f, w), first transform,
     // spectrum Z), then the W rows
-    ulonglong2 W[2 * S * WS];
-    float4 slot[2][NW];                  // candidates of the warps: maximum, shift offset, coefficient
+    ulonglong2 W[(Cfg<N>::TWICE ? 2 : 1) * S * Cfg<N>::WS];
+    float4 slot[2][N];                   // candidates of the warps: maximum, shift offset, coefficient
     float w0[S / 2 * S / 2];             // Eq. (5), one quadrant (symmetric)
     float wf[H1 * H1];                   // Eq. (9), one quadrant (symmetric)
     float2 cs[S];                        // cos, sin of 2 pi t / S
-    unsigned flags[NW];                  // per warp: 1 = a pixel of the support is available, 2 = an unknown target pixel
-    unsigned dmax[NW];
+    unsigned flags[N];                  // per warp: 1 = a pixel of the support is available, 2 = an unknown target pixel
+    unsigned dmax[N];
 };
 
-static_assert(2 * sizeof(float2) * S * AS <= sizeof(ulonglong2) * 2 * S * WS, "the transforms fit the W area");
+static_assert(2 * sizeof(float2) * S * AS <= sizeof(Smem<2>::W), "the transforms fit the W area");
 
 __device__ __forceinline__ int fold(int m) { return m < S / 2 ? m : S - 1 - m; }   // w0: m and S-1-m are alike
 __device__ __forceinline__ int foldf(int k) { return k <= S / 2 ? k : S - k; }      // w_f: k and S-k are alike
@@ -84,11 +99,15 @@ __device__ __forceinline__ int foldf(int k) { return k <= S / 2 ? k : S - k; }  
 // unrolled: a CTA that runs one block fetches this code cold, and the fetch is
 // most of its time.  The entries beyond one per thread go to another warp for
 // each table.
-__device__ __forceinline__ void tables(const MethodArgs& mth, Smem* sm) {
+template <int N>
+__device__ __forceinline__ void tables(const MethodArgs& mth, Smem<N>* sm) {
+    constexpr int T = Cfg<N>::T;
     const int tid = threadIdx.x;
     constexpr int EF = H1 * (H1 + 1) / 2;          // w_f: 153 pairs, rows r and 16 - r side by side
 #pragma unroll 1
-    for (int p = 0, i = tid; i < EF; i = ++p == 1 ? T + (tid + T - 32) % T : EF) {
+    for (int base = 0; base < EF; base += T) {
+        const int i = base + (base + T > EF ? (tid + T - 32) % T : tid);
+        if (i >= EF) continue;
         const int r = i / (H1 + 1), c = i % (H1 + 1);
         const bool first = c < H1 - r;
         const int m = first ? r : H1 - 1 - r, n = first ? r + c : c - 1;
@@ -96,7 +115,9 @@ __device__ __forceinline__ void tables(const MethodArgs& mth, Smem* sm) {
     }
     constexpr int H = S / 2, EW = H * (H + 1) / 2;   // w0: 136 pairs, rows r and 15 - r side by side
 #pragma unroll 1
-    for (int p = 0, i = tid; i < EW; i = ++p == 1 ? T + (tid + T - 64) % T : EW) {
+    for (int base = 0; base < EW; base += T) {
+        const int i = base + (base + T > EW ? (tid + T - 64) % T : tid);
+        if (i >= EW) continue;
         const int r = i / (H + 1), c = i % (H + 1);
         const bool first = c < H - r;
         const int m = first ? r : H - 1 - r, n = first ? r + c : c - 1;
@@ -131,64 +152,112 @@ __device__ __forceinline__ void butterfly_mj(float2& a, float2& b) {    // twidd
     a = make_float2(__fadd_rn(a.x, x.x), __fadd_rn(a.y, x.y));
 }
 
-// index of point i (bit-reversed position 8q + i) of warp q's 8 inputs
-__device__ __forceinline__ constexpr int in_index(int q2, int i) { return 4 * (((i & 1) << 2) | (i & 2) | (i >> 2)) + q2; }
+// the low `bits` bits of i reversed
+__device__ __forceinline__ constexpr int brev(int i, int bits) {
+    int r = 0;
+    for (int b = 0; b < bits; ++b) r |= ((i >> b) & 1) << (bits - 1 - b);
+    return r;
+}
+// index of point i of warp q (bit-reversed position PTS q + i); q2: q's bits reversed
+template <int N>
+__device__ __forceinline__ constexpr int in_index(int q2, int i) {
+    return N * brev(i, N == 4 ? 3 : 4) + q2;
+}
 
-// stages 1-3 on the 8 points of a thread, exchange through X, stages 4-5.
-// e[2 h + ..]: on return e[tt][p] is output t + 8 p, t = 2 q + tt.
-__device__ __forceinline__ void fft32_split(float2 (&x)[8], float2 (&e)[2][4], float2* X, const float2* cs, int q,
-                                            int lane) {
+// the first stages on the PTS points of a thread, exchange through X, the
+// last ones.  On return e[tt][p] is output TT q + tt + PTS p.
+template <int N>
+__device__ __forceinline__ void fft32_split(float2 (&x)[Cfg<N>::PTS], float2 (&e)[Cfg<N>::TT][N], float2* X,
+                                            const float2* cs, int q, int lane) {
+    constexpr int PTS = Cfg<N>::PTS, TT = Cfg<N>::TT;
 #pragma unroll
-    for (int i = 0; i < 8; i += 2) butterfly_one(x[i], x[i + 1]);
+    for (int half = 1; half < PTS; half *= 2)
 #pragma unroll
-    for (int i = 0; i < 8; i += 4) {
-        butterfly_one(x[i], x[i + 2]);
-        butterfly_mj(x[i + 1], x[i + 3]);
-    }
-    butterfly_one(x[0], x[4]);
-    butterfly(x[1], x[5], float(cos_2pi32(4)), float(-sin_2pi32(4)), 4);
-    butterfly_mj(x[2], x[6]);
-    butterfly(x[3], x[7], float(cos_2pi32(12)), float(-sin_2pi32(12)), 12);
+        for (int j = 0; j < PTS; j += 2 * half)
 #pragma unroll
-    for (int i = 0; i < 8; ++i) X[(8 * q + i) * AS + lane] = x[i];
+            for (int t = 0; t < half; ++t) {
+                const int tw = t * (16 / half);
+                if (tw == 0) butterfly_one(x[j + t], x[j + t + half]);
+                else if (tw == 8) butterfly_mj(x[j + t], x[j + t + half]);
+                else butterfly(x[j + t], x[j + t + half], float(cos_2pi32(tw)), float(-sin_2pi32(tw)), tw);
+            }
+#pragma unroll
+    for (int i = 0; i < PTS; ++i) X[(PTS * q + i) * AS + lane] = x[i];
     __syncthreads();
 #pragma unroll
-    for (int tt = 0; tt < 2; ++tt) {
-        const int t = 2 * q + tt;
+    for (int tt = 0; tt < TT; ++tt) {
+        const int t = TT * q + tt;
 #pragma unroll
-        for (int p = 0; p < 4; ++p) e[tt][p] = X[(t + 8 * p) * AS + lane];
-        const float2 c2 = cs[2 * t], c1 = cs[t], c9 = cs[t + 8];
-        butterfly(e[tt][0], e[tt][1], c2.x, -c2.y, 2 * t);
-        butterfly(e[tt][2], e[tt][3], c2.x, -c2.y, 2 * t);
-        butterfly(e[tt][0], e[tt][2], c1.x, -c1.y, t);
-        butterfly(e[tt][1], e[tt][3], c9.x, -c9.y, t + 8);
+        for (int p = 0; p < N; ++p) e[tt][p] = X[(t + PTS * p) * AS + lane];
+        const float2 c1 = cs[t];
+        if constexpr (N == 4) {
+            const float2 c2 = cs[2 * t], c9 = cs[t + 8];
+            butterfly(e[tt][0], e[tt][1], c2.x, -c2.y, 2 * t);
+            butterfly(e[tt][2], e[tt][3], c2.x, -c2.y, 2 * t);
+            butterfly(e[tt][0], e[tt][2], c1.x, -c1.y, t);
+            butterfly(e[tt][1], e[tt][3], c9.x, -c9.y, t + 8);
+        } else {
+            butterfly(e[tt][0], e[tt][1], c1.x, -c1.y, t);
+        }
     }
+}
+
+// A thread's lowest component holding its maximum mb, among the n components
+// o with values (r, i): the half that has it, the lower one first.
+template <int n>
+__device__ __forceinline__ void halve(const float (&o)[n], const float (&r)[n], const float (&i)[n], unsigned mb,
+                                      unsigned unit, unsigned& at, float& br, float& bi) {
+    if constexpr (n == 1) {
+        br = r[0];
+        bi = i[0];
+    } else {
+        float m = o[0];
+#pragma unroll
+        for (int j = 1; j < n / 2; ++j) m = fmaxf(m, o[j]);
+        const bool h = __float_as_uint(m) == mb;
+        float o2[n / 2], r2[n / 2], i2[n / 2];
+#pragma unroll
+        for (int j = 0; j < n / 2; ++j) {
+            o2[j] = h ? o[j] : o[j + n / 2];
+            r2[j] = h ? r[j] : r[j + n / 2];
+            i2[j] = h ? i[j] : i[j + n / 2];
+        }
+        at += h ? 0u : unit * (n / 2);
+        halve<n / 2>(o2, r2, i2, mb, unit, at, br, bi);
+    }
+}
+template <int n>
+__device__ __forceinline__ float max_of(const float (&o)[n]) {
+    if constexpr (n == 4) return fmaxf(max3(o[0], o[1], o[2]), o[3]);
+    else return max3(max3(o[0], o[1], o[2]), max3(o[3], o[4], o[5]), fmaxf(o[6], o[7]));
 }
 
 // One block by the whole CTA.  Every thread reaches every barrier.  BUILD: the
 // CTA's tables are built here, while the pixel loads are in flight.
-template <int B, bool REUSE, bool BUILD>
-__device__ __forceinline__ void block(const ImageArgs& im, int by, int bx, const MethodArgs& mth, Smem* sm,
+template <int B, int N, bool REUSE, bool BUILD>
+__device__ __forceinline__ void block(const ImageArgs& im, int by, int bx, const MethodArgs& mth, Smem<N>* sm,
                                       unsigned long long* empty, float delta) {
+    using C = Cfg<N>;
+    constexpr int T = C::T, G = C::G, NP = C::NP, WS = C::WS, PTS = C::PTS, TT = C::TT;
     constexpr int PT = (B * B + T - 1) / T;   // target pixels per thread
     const int tid = threadIdx.x, lane = tid & 31, q = tid >> 5;
     const int L = mth.L, y0 = by * B - L, x0 = bx * B - L;
     const long long blk = (long long)by * im.nbx + bx;
     int16_t* seq = im.seq ? im.seq + (size_t)blk * im.K : nullptr;
-    const int q2 = ((q & 1) << 1) | (q >> 1);   // the two bits of q reversed
+    const int q2 = N == 4 ? ((q & 1) << 1) | (q >> 1) : q;   // the bits of q reversed
     float2* X = reinterpret_cast<float2*>(sm->W);
     float2* A = X + S * AS;
 
-    // ---- a1: 8 pixels of column `lane` per thread, and the target pixels ----
-    float f[8];
+    // ---- a1: PTS pixels of column `lane` per thread, and the target pixels ----
+    float f[PTS];
     unsigned kn = 0, re = 0;
     {
         const int xc = x0 + lane;
         const bool xin = (unsigned)xc < (unsigned)im.W;
         const int pbx = xin ? xc / B : 0;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int y = y0 + in_index(q2, i);
+        for (int i = 0; i < PTS; ++i) {
+            const int y = y0 + in_index<N>(q2, i);
             bool known = false, reused = false;
             float fv = 0.f, pv = 0.f;
             if (xin && (unsigned)y < (unsigned)im.H) {
@@ -228,10 +297,10 @@ __device__ __forceinline__ void block(const ImageArgs& im, int by, int bx, const
     if constexpr (BUILD) tables(mth, sm);
     const unsigned avail = kn | re;
     __syncthreads();   // the tables are complete, the buffers free
-    float wv[8];
+    float wv[PTS];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const int m = in_index(q2, i);
+    for (int i = 0; i < PTS; ++i) {
+        const int m = in_index<N>(q2, i);
         const float w0 = sm->w0[fold(m) * (S / 2) + fold(lane)];
         // Eq. (5): w0 on known pixels, delta w0 on re-used ones, 0 elsewhere
         wv[i] = ((kn >> i) & 1u) ? w0 : (((re >> i) & 1u) ? delta * w0 : 0.f);
@@ -240,7 +309,8 @@ __device__ __forceinline__ void block(const ImageArgs& im, int by, int bx, const
     need = __reduce_or_sync(FULL, need | (avail ? 1u : 0u));
     if (lane == 0) sm->flags[q] = need;
     __syncthreads();
-    need = sm->flags[0] | sm->flags[1] | sm->flags[2] | sm->flags[3];
+    need = sm->flags[0] | sm->flags[1];
+    if constexpr (N == 4) need |= sm->flags[2] | sm->flags[3];
 
     float gacc[PT];
 #pragma unroll
@@ -264,10 +334,10 @@ __device__ __forceinline__ void block(const ImageArgs& im, int by, int bx, const
             sfw += __shfl_xor_sync(FULL, sfw, o);
         }
         const float mu = sfw / sw;
-        float2 x[8];
+        float2 x[PTS];
         unsigned dmax = 0;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
+        for (int i = 0; i < PTS; ++i) {
             const bool av = (avail >> i) & 1u;
             const float d = __fsub_rn(f[i], mu);
             x[i] = make_float2(av ? __fmul_rn(d, wv[i]) : 0.f, wv[i]);
@@ -277,35 +347,36 @@ __device__ __forceinline__ void block(const ImageArgs& im, int by, int bx, const
         dmax = __reduce_max_sync(FULL, dmax);
         if (lane == 0) sm->dmax[q] = dmax;
         __syncthreads();
-        dmax = max(max(sm->dmax[0], sm->dmax[1]), max(sm->dmax[2], sm->dmax[3]));
+        dmax = max(sm->dmax[0], sm->dmax[1]);
+        if constexpr (N == 4) dmax = max(dmax, max(sm->dmax[2], sm->dmax[3]));
         unsigned aexp = (dmax >> 23) + 1u;             // exponent field of alpha = 2^e
         aexp = (dmax >= 0x00800000u && dmax < 0x7e000000u) ? aexp : 127u;
         const float alpha = __uint_as_float(aexp << 23);
         const float inv2alpha = __uint_as_float((253u - aexp) << 23);   // 1 / (2 alpha)
 #pragma unroll
-        for (int i = 0; i < 8; ++i) x[i].y *= alpha;
+        for (int i = 0; i < PTS; ++i) x[i].y *= alpha;
 
         // ---- a3: over the rows (lane n = column n), then over the columns (lane k = row k) ----
 #pragma unroll 1
         for (int pass = 0; pass < 2; ++pass) {
-            float2 e[2][4];
-            fft32_split(x, e, X, sm->cs, q, lane);
+            float2 e[TT][N];
+            fft32_split<N>(x, e, X, sm->cs, q, lane);
             // first transform out by rows k, then back in by columns; the second stays transposed
             const int sk = pass == 0 ? AS : 1, sl = pass == 0 ? 1 : AS;
 #pragma unroll
-            for (int tt = 0; tt < 2; ++tt)
+            for (int tt = 0; tt < TT; ++tt)
 #pragma unroll
-                for (int p = 0; p < 4; ++p) A[(2 * q + tt + 8 * p) * sk + lane * sl] = e[tt][p];
+                for (int p = 0; p < N; ++p) A[(TT * q + tt + PTS * p) * sk + lane * sl] = e[tt][p];
             __syncthreads();
             if (pass == 0) {
 #pragma unroll
-                for (int i = 0; i < 8; ++i) x[i] = A[lane * AS + in_index(q2, i)];
+                for (int i = 0; i < PTS; ++i) x[i] = A[lane * AS + in_index<N>(q2, i)];
             }
         }
 
         // ---- Q and W of this thread's components ----
-        const int k = RPW * q + lane / G, g = lane % G;
-        f32x2 zr[NP], zi[NP], wf[NP], wur[NP], wui[NP];   // wu: the unshifted W row (DC phase)
+        const int k = C::RPW * q + lane / G, g = lane % G;
+        f32x2 zr[NP], zi[NP], wf[NP], wur[NP], wui[NP];   // wu: the unshifted W row
 #pragma unroll
         for (int j = 0; j < NP; ++j) {
             float qr[2], qi[2], wr[2], wi[2], f2[2];
@@ -335,8 +406,12 @@ __device__ __forceinline__ void block(const ImageArgs& im, int by, int bx, const
             const ulonglong2 e = make_ulonglong2(wur[j], wui[j]);
             const ulonglong2 x = make_ulonglong2(pack2(r1, r0), pack2(i1, i0));
             ulonglong2* w = sm->W + k * WS + g + G * j;
-            w[0] = w[S] = w[S * WS] = w[S * WS + S] = e;
-            w[S / 2] = w[S * WS + S / 2] = x;
+            w[0] = w[S] = e;
+            w[S / 2] = x;
+            if constexpr (C::TWICE) {
+                w[S * WS] = w[S * WS + S] = e;
+                w[S * WS + S / 2] = x;
+            }
         }
         __syncthreads();
         float w00, w16;
@@ -348,8 +423,13 @@ __device__ __forceinline__ void block(const ImageArgs& im, int by, int bx, const
             pm[p] = L + (tid + T * p) / B;
             pn[p] = L + (tid + T * p) % B;
         }
-        // W[k-u][l-v] lies u rows and v entries before this one
-        const ulonglong2* wbase = sm->W + (k + S) * WS + g + S;
+        // W[k-u][l-v], l = g
+        const ulonglong2* wbase = sm->W + (C::TWICE ? (k + S) * WS : 0) + g + S;
+        auto shifted = [&](unsigned o) {
+            if constexpr (C::TWICE) return wbase - o;   // u rows and v entries before W[k][g]
+            const int u = (int)((o * C::DIV) >> 16), v = (int)(o - (unsigned)u * WS);
+            return wbase + ((k - u) & (S - 1)) * WS - v;
+        };
         const unsigned off0 = (unsigned)(k * WS + g);
         float cr = 0.f, ci = 0.f;
         unsigned off;   // u * WS + v
@@ -369,31 +449,25 @@ __device__ __forceinline__ void block(const ImageArgs& im, int by, int bx, const
         // thread may publish is formed while the reductions run: its lowest
         // component holding its own maximum, by halving.
         auto pick = [&](int nu, const f32x2 (&vr)[NP], const f32x2 (&vi)[NP]) {
-            const float mlo = fmaxf(max3(olo[0], olo[1], olo[2]), olo[3]);
-            const float mhi = fmaxf(max3(ohi[0], ohi[1], ohi[2]), ohi[3]);
+            const float mlo = max_of(olo), mhi = max_of(ohi);
             const float m = fmaxf(mlo, mhi);
             const unsigned mb = __float_as_uint(m);
             const unsigned Mw = __reduce_max_sync(FULL, mb);
             target();   // of the previous pick
             const bool h1 = __float_as_uint(mlo) == mb;   // columns < 16
-            float o1[3], r1[NP], i1[NP];
+            float o1[NP], r1[NP], i1[NP], br, bi;
 #pragma unroll
             for (int j = 0; j < NP; ++j) {
                 float r0, rx, i0, ix;
                 unpack2(vr[j], r0, rx);
                 unpack2(vi[j], i0, ix);
-                if (j < 3) o1[j] = h1 ? olo[j] : ohi[j];
+                o1[j] = h1 ? olo[j] : ohi[j];
                 r1[j] = h1 ? r0 : rx;
                 i1[j] = h1 ? i0 : ix;
             }
-            const bool h2 = __float_as_uint(fmaxf(o1[0], o1[1])) == mb;   // of those the first two
-            const float o2 = h2 ? o1[0] : o1[2];
-            const float r20 = h2 ? r1[0] : r1[2], r21 = h2 ? r1[1] : r1[3];
-            const float i20 = h2 ? i1[0] : i1[2], i21 = h2 ? i1[1] : i1[3];
-            const bool h3 = __float_as_uint(o2) == mb;
-            const float br = h3 ? r20 : r21, bi = h3 ? i20 : i21;
             // index u * S + v as the offset u * WS + v: the same order
-            const unsigned boff = off0 + (h1 ? 0u : S / 2) + (h2 ? 0u : 2u * G) + (h3 ? 0u : (unsigned)G);
+            unsigned boff = off0 + (h1 ? 0u : S / 2);
+            halve<NP>(o1, r1, i1, mb, (unsigned)G, boff, br, bi);
             const unsigned lo = __reduce_min_sync(FULL, mb == Mw ? boff : 0xffffffffu);
             // c = gamma p (Eq. 10)
             const float4 mine = make_float4(m, __uint_as_float(boff), br * cg, bi * cg);
@@ -401,11 +475,17 @@ __device__ __forceinline__ void block(const ImageArgs& im, int by, int bx, const
             if (mb == Mw && boff == lo) sl[q] = mine;
             __syncthreads();   // one barrier per iteration: the slots alternate
             // rows ascend with the warp, so the first maximum has the lowest index
-            float4 c0 = sl[0], c2 = sl[2];
-            const float4 c1 = sl[1], c3 = sl[3];
-            if (__float_as_uint(c1.x) > __float_as_uint(c0.x)) c0 = c1;
-            if (__float_as_uint(c3.x) > __float_as_uint(c2.x)) c2 = c3;
-            if (__float_as_uint(c2.x) > __float_as_uint(c0.x)) c0 = c2;
+            float4 c0 = sl[0];
+            const float4 c1 = sl[1];
+            if constexpr (N == 4) {
+                float4 c2 = sl[2];
+                const float4 c3 = sl[3];
+                if (__float_as_uint(c1.x) > __float_as_uint(c0.x)) c0 = c1;
+                if (__float_as_uint(c3.x) > __float_as_uint(c2.x)) c2 = c3;
+                if (__float_as_uint(c2.x) > __float_as_uint(c0.x)) c0 = c2;
+            } else {
+                if (__float_as_uint(c1.x) > __float_as_uint(c0.x)) c0 = c1;
+            }
             off = __float_as_uint(c0.y);
             cr = c0.z;
             ci = c0.w;
@@ -415,7 +495,7 @@ __device__ __forceinline__ void block(const ImageArgs& im, int by, int bx, const
         // (in every thread: a branch to the warps that have target pixels costs
         // 50 cycles of the iteration)
         auto note = [&](int nu, auto rec) {
-            const int u = (int)((off * kDivWS) >> 16), v = (int)(off - (unsigned)u * WS);
+            const int u = (int)((off * C::DIV) >> 16), v = (int)(off - (unsigned)u * WS);
             if constexpr (rec.value) {
                 if (tid == 0) seq[nu] = (int16_t)(u * S + v);
             }
@@ -454,17 +534,22 @@ __device__ __forceinline__ void block(const ImageArgs& im, int by, int bx, const
             }
             for (;;) {   // the pick of iteration nu is not applied yet
                 if (nu + 1 == K) break;
-                const ulonglong2* row = wbase - off;   // a7 (Eq. 12) and the next objective
-                ulonglong2 w[NP];
-#pragma unroll
-                for (int j = 0; j < NP; ++j) w[j] = row[G * j];
-                note(nu++, rec);   // while the loads are under way
+                const ulonglong2* row = shifted(off);   // a7 (Eq. 12) and the next objective
                 const f32x2 ncr2 = pack2(-cr, -cr), ci2 = pack2(ci, ci), nci2 = pack2(-ci, -ci);
+                constexpr int NL = 4;
 #pragma unroll
-                for (int j = 0; j < NP; ++j) {
-                    zr[j] = ffma2(ncr2, w[j].x, ffma2(ci2, w[j].y, zr[j]));
-                    zi[j] = ffma2(ncr2, w[j].y, ffma2(nci2, w[j].x, zi[j]));
-                    unpack2(objective2(zr[j], zi[j], wf[j]), olo[j], ohi[j]);
+                for (int j0 = 0; j0 < NP; j0 += NL) {
+                    ulonglong2 w[NL];
+#pragma unroll
+                    for (int j = 0; j < NL; ++j) w[j] = row[G * (j0 + j)];
+                    if (j0 == 0) note(nu++, rec);   // while the loads are under way
+#pragma unroll
+                    for (int j = 0; j < NL; ++j) {
+                        f32x2 &a = zr[j0 + j], &b = zi[j0 + j];
+                        a = ffma2(ncr2, w[j].x, ffma2(ci2, w[j].y, a));
+                        b = ffma2(ncr2, w[j].y, ffma2(nci2, w[j].x, b));
+                        unpack2(objective2(a, b, wf[j0 + j]), olo[j0 + j], ohi[j0 + j]);
+                    }
                 }
                 pick(nu, zr, zi);
             }
@@ -489,15 +574,15 @@ __device__ __forceinline__ void block(const ImageArgs& im, int by, int bx, const
 // One block per CTA, the grid sized to the work.  INLINE: one image whose
 // arguments are kernel parameters; else images and block prefix sums of a
 // work table in device memory.
-template <int B, bool INLINE>
-__global__ void __launch_bounds__(T) fsr_coop_kernel(const __grid_constant__ BatchArgs a,
+template <int B, int N, bool INLINE>
+__global__ void __launch_bounds__(Cfg<N>::T, Cfg<N>::MIN_CTAS) fsr_coop_kernel(const __grid_constant__ BatchArgs a,
                                                      const __grid_constant__ ImageArgs one) {
     extern __shared__ __align__(16) unsigned char smem[];
-    Smem* sm = reinterpret_cast<Smem*>(smem);
+    Smem<N>* sm = reinterpret_cast<Smem<N>*>(smem);
     const long long item = blockIdx.x;
     if constexpr (INLINE) {
         const int by = (int)item / one.nbx;
-        block<B, false, true>(one, by, (int)item - by * one.nbx, a.mth, sm, a.empty, 0.f);
+        block<B, N, false, true>(one, by, (int)item - by * one.nbx, a.mth, sm, a.empty, 0.f);
     } else {
         int lo = 0, hi = a.n - 1;   // image of this entry: last i with first[i] <= item
         while (lo < hi) {
@@ -508,15 +593,15 @@ __global__ void __launch_bounds__(T) fsr_coop_kernel(const __grid_constant__ Bat
         const ImageArgs im = a.images[lo];
         const int blk = (int)(item - __ldg(a.first + lo));
         const int by = blk / im.nbx;
-        block<B, false, true>(im, by, blk - by * im.nbx, a.mth, sm, a.empty, 0.f);
+        block<B, N, false, true>(im, by, blk - by * im.nbx, a.mth, sm, a.empty, 0.f);
     }
 }
 
 // Re-use form: one launch per wavefront (see fsr_reuse_kernel), a CTA per block.
 template <int B, int NSEG>
-__global__ void __launch_bounds__(T) fsr_coop_reuse_kernel(const __grid_constant__ ReuseLaunchN<NSEG> a) {
+__global__ void __launch_bounds__(Cfg<4>::T) fsr_coop_reuse_kernel(const __grid_constant__ ReuseLaunchN<NSEG> a) {
     extern __shared__ __align__(16) unsigned char smem[];
-    Smem* sm = reinterpret_cast<Smem*>(smem);
+    Smem<4>* sm = reinterpret_cast<Smem<4>*>(smem);
     tables(a.mth, sm);
     // a programmatic dependent of the previous wavefront: nothing of the
     // image or the output is read before that one has completed
@@ -529,7 +614,7 @@ __global__ void __launch_bounds__(T) fsr_coop_reuse_kernel(const __grid_constant
     }
     const ReuseSeg& sg = a.seg[s];
     const int by = sg.by_lo + (j - sg.first);
-    block<B, true, false>(sg.im, by, a.t - a.slope * by, a.mth, sm, a.empty, a.delta);
+    block<B, 4, true, false>(sg.im, by, a.t - a.slope * by, a.mth, sm, a.empty, a.delta);
 }
 
 // Re-use form in one launch: a CTA takes block rows in order and works through
@@ -591,10 +676,10 @@ __device__ __forceinline__ bool row_wait(const unsigned long long* slot, unsigne
 }
 
 template <int B>
-__global__ void __launch_bounds__(T) fsr_coop_rows_kernel(const __grid_constant__ RowsArgs a) {
+__global__ void __launch_bounds__(Cfg<4>::T) fsr_coop_rows_kernel(const __grid_constant__ RowsArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_row, s_ok;
-    Smem* sm = reinterpret_cast<Smem*>(smem);
+    Smem<4>* sm = reinterpret_cast<Smem<4>*>(smem);
     tables(a.mth, sm);
     for (;;) {
         if (threadIdx.x == 0) s_row = (int)atomicAdd(a.ring + kRowRing, 1ull);
@@ -627,7 +712,7 @@ __global__ void __launch_bounds__(T) fsr_coop_rows_kernel(const __grid_constant_
         __syncthreads();
         for (int bx = 0; bx < im.nbx; ++bx) {
             // the row above, while thread 0 publishes the last block
-            if (threadIdx.x == T - 1 && r > 0 && s_ok &&
+            if (threadIdx.x == Cfg<4>::T - 1 && r > 0 && s_ok &&
                 !row_wait(a.ring + prev % kRowRing, (unsigned)prev, (unsigned)min(bx + a.lag, im.nbx), limit))
                 s_ok = 0;
             __syncthreads();
@@ -635,7 +720,7 @@ __global__ void __launch_bounds__(T) fsr_coop_rows_kernel(const __grid_constant_
                 if (threadIdx.x == 0) atomicOr(a.status, kStatusRowWait);
                 return;
             }
-            block<B, true, false>(im, r, bx, a.mth, sm, a.empty, a.delta);
+            block<B, 4, true, false>(im, r, bx, a.mth, sm, a.empty, a.delta);
             __syncthreads();
             // (release at the end of a barrier: the CTA's pixels come before it)
             if (threadIdx.x == 0) st_release(slot, tag | (bx + 1 == im.nbx ? 0xffffffffu : (unsigned)(bx + 1)));

@@ -17,7 +17,7 @@ cudaError_t configure_fp32_batch() {
 cudaError_t launch_batch_fp32(const BatchArgs& a, int B, Schedule sc, int sm_count, cudaStream_t stream) {
     if (sc.warps != kWarpsFp32) return launch_batch_fp32_sched(a, B, sc, sm_count, stream);
     // few blocks: a CTA per block (no tile copies, so not when the test hook arms one)
-    if (a.total <= (long long)kCoopBlocksPerSm * sm_count && a.tx_extra == 0) return launch_coop(a, B, nullptr, stream);
+    if (a.total <= (long long)kCoopBlocksPerSm * sm_count && a.tx_extra == 0) return launch_coop(a, B, nullptr, sm_count, stream);
     switch (B) {
         case 2: return launch_batch_t<float, 2, kWarpsFp32>(a, sm_count, stream);
         case 4: return launch_batch_t<float, 4, kWarpsFp32>(a, sm_count, stream);

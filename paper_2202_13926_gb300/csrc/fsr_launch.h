@@ -48,28 +48,34 @@ cudaError_t launch_batch_small(const BatchArgs& a, int S, int B, int fp64, int c
                                cudaStream_t stream);
 
 // CTA-per-block FP32 kernels of S = 32 (fsr_coop.cuh), for launches of few
-// blocks.  A block that has an SM (nearly) to itself is done in half the time
-// of the one-warp kernel; with more of them the four warps of a block cost
-// more issue slots than its one warp does.  The lines, measured:
-//   independent blocks, us per call, one-warp / CTA-per-block kernel: 0.4
-//   blocks per SM K = 100 75 / 29, 2.2 74 / 41, 3.8 73 / 49, 4.4 74 / 68, 5.9
-//   74 / 74 (K = 25 35 / 33), 6.7 74 / 82 (K = 25 35 / 35);
-//   re-use form, K = 50, ms for n 1080p frames together with the line at 0, 4,
-//   6, 8, 10, 16 blocks per SM: n = 8 98, 82, 68, 68, 68, 69; n = 16 103, 97,
-//   95, 94, 96, 113; n = 24 120, 115, 114, 113, 115, 160.
+// blocks: four warps per block up to kCoop4BlocksPerSm blocks per SM, two up to
+// kCoopBlocksPerSm, then the one-warp kernel.  A block that has an SM (nearly)
+// to itself is done in a third of the one-warp kernel's time; with more of them
+// the warps of a block cost more issue slots than one warp does.  Independent
+// blocks, us per call with four / two warps / one warp, K = 100 (K = 25): 0.4
+// blocks per SM 27 / 27 / 75; 2.2 39 / 43 / 74; 3.8 47 / 45 / 73; 4.4 64 (29) /
+// 58 (25) / 74 (35); 6.7 78 / 70 / 74 (33 / 29 / 35); 8.1 102 / 90 / 102; 10.5
+// 109 / 103 / 110 (48 / 43 / 47); 13.3 110 / 117 / 108.
+// A wavefront of the re-use form takes four warps per block up to
+// kCoopReusePerSm blocks per SM (K = 50, ms for n 1080p frames together with
+// the line at 0, 4, 6, 8, 10, 16: n = 8 98, 82, 68, 68, 68, 69; n = 16 103, 97,
+// 95, 94, 96, 113; n = 24 120, 115, 114, 113, 115, 160).
 // `one`: a single image as kernel parameters (no work table), or nullptr for
 // the table of a.
-constexpr int kCoopBlocksPerSm = 6;
+constexpr int kCoop4BlocksPerSm = 3;
+constexpr int kCoopBlocksPerSm = 11;
 constexpr int kCoopReusePerSm = 8;
 cudaError_t configure_coop();
-cudaError_t launch_coop(const BatchArgs& a, int B, const ImageArgs* one, cudaStream_t stream);
+cudaError_t launch_coop(const BatchArgs& a, int B, const ImageArgs* one, int sm_count, cudaStream_t stream);
+cudaError_t configure_coop2();
+cudaError_t launch_coop2(const BatchArgs& a, int B, const ImageArgs* one, cudaStream_t stream);
 cudaError_t launch_coop_reuse(const ReuseLaunch& a, int B, cudaStream_t stream);
 // Re-use form in one launch (fsr_coop_rows_kernel), for calls with at most
 // kCoopRowsPerSm block rows at work per SM (ms, a launch per wavefront / one
-// launch: one 1080p frame, K = 100 53.5 / 45.3; n of them, K = 50: n = 8 (5.1
-// rows per SM) 69.4 / 57.1, 12 (7.7) 88.0 / 78.0, 16 (10.2) 94.3 / 97.4, 24
-// 113 / 142), over `ring`, device memory
-// of coop_rows_bytes() that no other launch uses meanwhile.
+// launch: one 1080p frame, K = 100 53.5 / 45.3, now 40.8; n of them, K = 50: n =
+// 8 (5.1 rows per SM) 69.4 / 57.1, 12 (7.7) 88.0 / 78.0, 16 (10.2) 94.3 / 97.4,
+// 24 113 / 142), over `ring`, device memory of coop_rows_bytes() that no other
+// launch uses meanwhile.
 // coop_rows_parallel: the block rows that can be at work at once (the
 // wavefronts' width; 2^31 - 1 for more images than a launch takes).
 constexpr int kCoopRowsPerSm = 8;

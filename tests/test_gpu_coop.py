@@ -1,7 +1,7 @@
 """The CTA-per-block FP32 kernel (few blocks in a launch) against the one-warp
 kernel: same arithmetic, so images, selected indices and empty-block counts
 are equal bit for bit.  The one-warp kernel runs the same image when a second
-image lifts the launch above the line (4 blocks per SM)."""
+image lifts the launch above the line."""
 import numpy as np
 import pytest
 
@@ -24,9 +24,11 @@ def handle():
     h.close()
 
 
-# one block; ragged in both directions; the last size below the line at B = 4
-# on 152 SMs (608 blocks) and the first above it
-SIZES = [(3, 2, 4), (33, 47, 2), (61, 83, 4), (64, 152, 4), (64, 156, 4), (97, 101, 8), (131, 90, 16)]
+# one block; ragged in both directions; at B = 4 on 152 SMs the last size of the
+# four-warp form (456 blocks), the first and the last of the two-warp form (475,
+# 1672) and the first of the one-warp kernel; two warps at the other B
+SIZES = [(3, 2, 4), (33, 47, 2), (61, 83, 4), (76, 96, 4), (76, 97, 4), (152, 176, 4), (152, 177, 4), (97, 101, 8),
+         (131, 90, 16), (50, 61, 2), (203, 239, 8), (399, 470, 16)]
 
 
 @pytest.mark.parametrize("H,W,B", SIZES)
@@ -42,8 +44,8 @@ def test_cta_per_block_equals_one_warp(handle, H, W, B, mask_kind, K, opts):
     m = torch.from_numpy(mask).to(dev)
     n = -(-H // B) * -(-W // B)
     border = (32 - B) // 2
-    big = torch.zeros(256, 640, device=dev)
-    big_mask = torch.ones(256, 640, dtype=torch.uint8, device=dev)
+    big = torch.zeros(512, 1280, device=dev)
+    big_mask = torch.ones(512, 1280, dtype=torch.uint8, device=dev)
 
     def run(extra, batch):
         out = torch.full((H, W), -7.0, device=dev)
