@@ -619,30 +619,32 @@ constexpr int WS32 = WRow<float>::stride;
 // Groups per row: the group holding the maximum is published, so more groups
 // mean fewer stores and more to search.  1080p, K = 100, ms per frame with the
 // pick by reductions: 2 groups 4.82, 4 groups 4.65, 8 groups 4.78 (2 groups
-// and ballots: 4.84).
-constexpr int NG = 4;            // groups per row
-constexpr int GS = S / NG;       // components per group
-static_assert(GS % 4 == 0 && GS <= 16, "a group is published as GS / 4 float4 stores");
+// and ballots: 4.84).  With the pair update 4 groups are the slower ones: 7.24
+// and 7.41 (2 groups and ballots: 7.27).
+template <bool CONJ>
+constexpr int kGroups = CONJ ? 2 : 4;
 
 __device__ __forceinline__ float wf_at(const float (&wfr)[S / 2 + 1], int l) {
     return wfr[l <= S / 2 ? l : S - l];
 }
 
+template <int NG>
 __device__ __forceinline__ void group_max(float (&g)[NG], int i, float o0, float o1) {
-    // pair i = components 2i, 2i+1 belongs to group i / (GS / 2)
-    constexpr int PPG = GS / 2;
+    // pair i = components 2i, 2i+1 belongs to group i / (S / NG / 2)
+    constexpr int PPG = S / NG / 2;
     if (i % PPG == 0) g[i / PPG] = fmaxf(o0, o1);
     else g[i / PPG] = max3(g[i / PPG], o0, o1);
 }
 
 // maximum over the groups
+template <int NG>
 __device__ __forceinline__ float groups_max(const float (&g)[NG]) {
-    if constexpr (NG == 8) return max3(max3(g[0], g[1], g[2]), max3(g[3], g[4], g[5]), fmaxf(g[6], g[7]));
-    else if constexpr (NG == 4) return fmaxf(max3(g[0], g[1], g[2]), g[3]);
+    if constexpr (NG == 4) return fmaxf(max3(g[0], g[1], g[2]), g[3]);
     else return fmaxf(g[0], g[1]);
 }
 
 // objective pass of R = a W + Q over the unshifted row k (DC phase)
+template <int NG>
 __device__ __forceinline__ void pass_split_objective(const float (&zr)[S], const float (&zi)[S],
                                                      const float (&wfr)[S / 2 + 1], const float2* wrow,
                                                      float ar, float ai, float (&g)[NG]) {
@@ -676,7 +678,7 @@ __device__ __forceinline__ void pass_fold(float (&zr)[S], float (&zi)[S], const 
 // 48-entry row.  For odd offsets the 16-byte loads start one entry earlier
 // and each component takes the upper half of one load and the lower half of
 // the next.
-template <bool ODD>
+template <bool ODD, int NG>
 __device__ __forceinline__ void half_update(float (&zr)[S], float (&zi)[S], const float (&wfr)[S / 2 + 1],
                                             const float2* base, int h, float cr, float ci, float (&g)[NG]) {
     const float4* p = reinterpret_cast<const float4*>(ODD ? base - 1 : base);
@@ -700,7 +702,7 @@ __device__ __forceinline__ void half_update(float (&zr)[S], float (&zi)[S], cons
     }
 }
 
-template <bool ODD>
+template <bool ODD, int NG>
 __device__ __forceinline__ void pass_update(float (&zr)[S], float (&zi)[S], const float (&wfr)[S / 2 + 1],
                                             const float2* row, int s, float cr, float ci, float (&g)[NG]) {
     half_update<ODD>(zr, zi, wfr, row + s, 0, cr, ci, g);
@@ -719,7 +721,7 @@ __device__ __forceinline__ void pair_update(float& re, float& im, float w1r, flo
     im = fma_rn(-cr, si, fma_rn(-ci, dr, im));
 }
 
-template <bool ODD>
+template <bool ODD, int NG>
 __device__ __forceinline__ void half_update_pair(float (&zr)[S], float (&zi)[S], const float (&wfr)[S / 2 + 1],
                                                  const float2* base1, const float2* base2, int h, float cr,
                                                  float ci, float (&g)[NG]) {
@@ -750,7 +752,7 @@ __device__ __forceinline__ void half_update_pair(float (&zr)[S], float (&zi)[S],
 
 // Row k reads row1 = W[k-u] from column s1 = -v and row2 = W[k+u] from
 // column s2 = v (mod 32); s1 and s2 have the parity of v.
-template <bool ODD>
+template <bool ODD, int NG>
 __device__ __forceinline__ void pass_update_pair(float (&zr)[S], float (&zi)[S], const float (&wfr)[S / 2 + 1],
                                                  const float2* row1, int s1, const float2* row2, int s2,
                                                  float cr, float ci, float (&g)[NG]) {
@@ -781,11 +783,13 @@ __device__ __forceinline__ void st_shared_64(uint32_t addr, bool p, float a0, fl
         : "memory");
 }
 
-// Lane u writes components GS*j .. GS*j+GS-1 of its row to rowbuf[0..GS-1]
-// (j uniform).
-template <int J>
+// Lane u writes components GS*j .. GS*j+GS-1 (GS = S / NG) of its row to
+// rowbuf[0..GS-1] (j uniform).
+template <int NG, int J>
 __device__ __forceinline__ void store_group(const float (&zr)[S], const float (&zi)[S], float4* pub) {
     if constexpr (J < NG) {
+        constexpr int GS = S / NG;
+        static_assert(GS % 4 == 0 && GS <= 16, "a group is published as GS / 4 float4 stores");
 #pragma unroll
         for (int t = 0; t < GS / 2; ++t) {
             const int c = GS * J + 2 * t;
@@ -794,16 +798,16 @@ __device__ __forceinline__ void store_group(const float (&zr)[S], const float (&
     }
 }
 
+template <int NG>
 __device__ __forceinline__ void publish_group(const float (&zr)[S], const float (&zi)[S], int j,
                                               bool mine, float2* rowbuf) {
     float4* pub = reinterpret_cast<float4*>(rowbuf);
     switch (j) {
 #define FSR_PUB_CASE(J)                               \
         case J:                                       \
-            if (mine) store_group<J>(zr, zi, pub);    \
+            if (mine) store_group<NG, J>(zr, zi, pub);    \
             break;
         FSR_PUB_CASE(0) FSR_PUB_CASE(1) FSR_PUB_CASE(2) FSR_PUB_CASE(3)
-        FSR_PUB_CASE(4) FSR_PUB_CASE(5) FSR_PUB_CASE(6) FSR_PUB_CASE(7)
 #undef FSR_PUB_CASE
         default: break;
     }
@@ -816,10 +820,11 @@ struct Pick {
     float Rr, Ri;
 };
 
-template <bool SPLIT>
+template <bool SPLIT, int NG>
 __device__ __forceinline__ Pick argmax_pick(const float (&zr)[S], const float (&zi)[S], const float (&g)[NG],
                                             const float2* Wd, float2* rowbuf, const float* __restrict__ swf,
                                             float ar, float ai, int lane) {
+    constexpr int GS = S / NG;
     const float m = groups_max(g);
     const unsigned Mb = __reduce_max_sync(FULL, __float_as_uint(m));
     // the lowest (row, group of the row) holding it, by a second reduction: a
@@ -829,7 +834,7 @@ __device__ __forceinline__ Pick argmax_pick(const float (&zr)[S], const float (&
     for (int j = NG - 1; j >= 0; --j) c0 = __float_as_uint(g[j]) == Mb ? (unsigned)(NG * lane + j) : c0;
     const unsigned cm = __reduce_min_sync(FULL, c0);
     const int u = (int)(cm / NG) & (S - 1), jg = (int)(cm % NG);
-    publish_group(zr, zi, jg, lane == u, rowbuf);
+    publish_group<NG>(zr, zi, jg, lane == u, rowbuf);
     __syncwarp();
     const int cl = GS * jg + (lane & (GS - 1));   // column examined by this lane
     const float2 q = rowbuf[lane & (GS - 1)];
@@ -911,7 +916,7 @@ __device__ __forceinline__ void iterate(float (&zr)[S], float (&zi)[S], float2* 
     }
     const float cg = gamma * (1.f / st.W0);
     const float2* wrow_k = Wd + lane * WS32;
-    float g[NG];
+    float g[kGroups<CONJ>];
     float cr, ci;
     Pick pk;
     int nu = 0;
@@ -1282,7 +1287,10 @@ __device__ __forceinline__ unsigned scan_targets(const BatchArgs& a, long long b
 }
 
 // Batch form: every warp takes consecutive entries of the block list
-// (guided_take) at a time; images are ordered by decreasing K so the long blocks start first.
+// (guided_take) at a time; images are ordered by decreasing K so the long
+// blocks start first.  With the pair update it takes `chunk` at a time: the
+// guided share's code around it costs the iteration registers (7.24 -> 7.45 ms
+// per 1080p frame at K = 100).
 // ONE_ROUND: short-lived CTAs (a warp takes one chunk; the grid is sized to
 // the work), used by the serving loop so that the CTAs of a launch on a
 // higher-priority stream are scheduled as soon as running CTAs finish.
@@ -1316,7 +1324,7 @@ fsr_batch_kernel(const BatchArgs a) {
     const T gamma = T(a.mth.gamma);
     long long seen = 0;   // entries taken by all warps, as of this warp's last take
     for (;;) {
-        const int take = ONE_ROUND ? a.chunk : guided_take(a, seen, (int)gridDim.x * WARPS, a.chunk);
+        const int take = ONE_ROUND || CONJ ? a.chunk : guided_take(a, seen, (int)gridDim.x * WARPS, a.chunk);
         unsigned long long base = 0;
         if (lane == 0) base = atomicAdd(a.counter, (unsigned long long)take);
         base = __shfl_sync(FULL, base, 0);
