@@ -1,6 +1,6 @@
 // FP32 FSR with a support S in {8, 16} (B <= S; the support-size study of Sec.
-// IV, Figs. 3 and 5; S = 4: fsr_quad.cu): one group of S lanes per block, 32 / S blocks per
-// warp.  Lane t of a group holds column t of the support, then row t of the
+// IV, Figs. 3 and 5; S = 4: fsr_quad.cu): one group of S lanes per block, 32 / S
+// blocks per warp.  Lane t of a group holds column t of the support, then row t of the
 // spectrum (S complex values in registers), as the S = 32 kernel does with a
 // whole warp:
 //   a1-a3  the support is loaded by columns, the weighted mean mu is removed,
@@ -18,8 +18,8 @@
 //          half-warp on distinct bank pairs; the objective of Eq. (8) is
 //          rounded explicitly; the lane holding the block maximum publishes
 //          its row in shared memory and lane t of the group forms the
-//          objective of component t again, so the lowest index with the
-//          maximum is found by two ballots;
+//          objective of component t again; the lowest index with the
+//          maximum is found by reductions and ballots;
 //   a9     Re g (sparse inverse of G) accumulated at the target pixels only.
 // The blocks of a warp may have different K and leave the DC phase at
 // different iterations: the loop runs to the largest K and every step that is

@@ -72,7 +72,7 @@ cudaError_t launch_coop2(const BatchArgs& a, int B, const ImageArgs* one, cudaSt
 cudaError_t launch_coop_reuse(const ReuseLaunch& a, int B, cudaStream_t stream);
 // Re-use form in one launch (fsr_coop_rows_kernel), for calls with at most
 // kCoopRowsPerSm block rows at work per SM (ms, a launch per wavefront / one
-// launch: one 1080p frame, K = 100 53.5 / 45.3, now 40.8; n of them, K = 50: n =
+// launch: one 1080p frame, K = 100 53.5 / 45.3, now 39.6; n of them, K = 50: n =
 // 8 (5.1 rows per SM) 69.4 / 57.1, 12 (7.7) 88.0 / 78.0, 16 (10.2) 94.3 / 97.4,
 // 24 113 / 142), over `ring`, device memory of coop_rows_bytes() that no other
 // launch uses meanwhile.

@@ -27,9 +27,10 @@
 // (exactly Hermitian, as in the oracle).
 //
 // Measured (K = 100, B = 4), 4 lanes per block -> this: 1280 x 720 133 -> 94 us,
-// 480 x 480 72 -> 50 us, 64 x 64 48 -> 43 us; 350 -> 290 instructions per warp
-// and iteration, of 8 blocks then and of 32 now.  What bounds it now: the latency
-// of one iteration's chain (0.4 us) at 3 warps per scheduler.
+// 480 x 480 72 -> 50 us, 64 x 64 48 -> 43 us, 1080p 250 -> 182 us; 16.1 -> 10.7
+// instructions per block and iteration (129 per warp, of 8 blocks, then; 344, of
+// 32, now).  What bounds it now: the issue slots and the latency of one
+// iteration's chain (0.4 us) at 3 warps per scheduler (issue active 66 %).
 #include "fsr_launch.h"
 
 namespace fsrk {

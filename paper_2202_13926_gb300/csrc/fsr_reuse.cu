@@ -2,8 +2,12 @@
 // that Sec. II leaves out): the wavefront kernel, FP32 and FP64, every B of
 // the 32 x 32 support.  One warp per block of the wavefront (the launch
 // shapes are in fsr_reuse.cuh), or for FP32 wavefronts of few blocks a CTA
-// per block (fsr_coop.cuh): one 1080p frame, K = 100, delta = 0.5: 104.0 ->
-// 53.5 ms, six 480 x 270 frames 27.6 -> 14.7 ms, bit-identical.
+// per block (fsr_coop.cuh): 16 1080p frames, K = 50: 103 -> 95 ms, 24: 120 ->
+// 114 ms.  FP32 calls of few block rows take one launch for all wavefronts
+// (fsr_coop_rows_kernel) unless they are captured: one 1080p frame, K = 100:
+// 104.0 ms with a warp per block, 53.5 with a CTA per block and a launch per
+// wavefront, 45.2 in one launch, 39.6 since its iteration is packed; six
+// 480 x 270 frames 27.6, 14.7, 11.3 and 9.9 ms; all bit-identical.
 #include "fsr_reuse.cuh"
 
 namespace fsrk {

@@ -112,7 +112,8 @@ struct Layout {
 // Warps per CTA: 8; FP64 at S = 24 takes 4 (shared memory per warp).  FP32
 // at S = 24 runs one CTA of 20 warps per SM (at most 96 registers; 220 KB of
 // shared memory): 1080p, K = 100, B = 4: 4.52 ms with 2 CTAs x 8 warps (at
-// most 128 registers), 4.31 ms with 18 warps, 4.20 ms with 20.
+// most 128 registers), 4.31 ms with 18 warps, 4.20 ms with 20 (3.99 ms since the
+// published values go out in predicated stores).
 template <typename T, int SZ>
 constexpr int warps() { return (sizeof(T) == 8 && SZ == 24) ? 4 : (SZ == 24 ? 20 : 8); }
 
