@@ -100,10 +100,12 @@ typedef struct fsr_params {
                          FSR: blocks in raster order, and an unknown pixel of an earlier
                          block's target takes part in later supports with its
                          reconstruction and the weight delta * rho^dist of Eq. (5).
-                         Runs as one launch per wavefront of blocks (t = a*by + bx,
-                         a = ceil(L/B) + 1); fsr_reconstruct, fsr_reconstruct_host and
-                         fsr_reconstruct_batch (each image its own raster order, the
-                         images sharing the wavefront launches), S = 32,
+                         FSR_FP32 calls of few block rows run as one launch whose block
+                         rows follow each other (not under stream capture); the others
+                         as one launch per wavefront of blocks (t = a*by + bx,
+                         a = ceil(L/B) + 1).  The results are the same.  fsr_reconstruct,
+                         fsr_reconstruct_host and fsr_reconstruct_batch (each image its
+                         own raster order, the images sharing the launches), S = 32,
                          FSR_UPDATE_SINGLE, FSR_FP32 / FSR_FP64_DEBUG only. */
 } fsr_params;
 
@@ -155,17 +157,19 @@ int fsr_reconstruct_host(fsr_handle *h, const float *img, const uint8_t *mask,
                          float *out, void *stream);
 
 /* Support tiles (step a1 of every block, Sec. III-A, Eq. 13): when img and
- * mask are 16-byte aligned and pitch is a multiple of 16, the single-image
+ * mask are 16-byte aligned and pitch is a multiple of 16, the one-warp
  * kernels bring each block's 32 x 32 support in by two TMA tile copies (the
  * image and the mask), with pixels outside the image filled as unknown;
- * otherwise by plain loads.  Both give identical results.  A warp waits for
+ * otherwise, and in FSR_FP32 calls of few blocks (up to 11 per SM, which a CTA
+ * per block computes), by plain loads.  All give identical results.  A warp waits for
  * its copies with a bounded wait (about one second); when the wait gives up,
  * the warp sets a bit in the handle's device status word and takes no more
  * blocks (their output pixels are left unwritten).
  *
  * fsr_check_status synchronises `stream`, then reads and clears the status
  * word: FSR_OK, or FSR_ERR_TIMEOUT with a message when a wait gave up in any
- * single-image launch on h since the last check.  fsr_reconstruct_host does
+ * single-image launch on h since the last check (a tile copy's, or in the re-use
+ * form that of a block row for the row above it, bounded in the same way).  fsr_reconstruct_host does
  * this check itself.  Errors: INVALID_ARG (h NULL), CUDA. */
 int fsr_check_status(fsr_handle *h, void *stream);
 
@@ -192,9 +196,11 @@ long long fsr_num_blocks(int height, int width, int block);
 /* ---- Batch form: many images in one persistent launch ------------------
  * The blocks of all images form one work list, images ordered by decreasing
  * K (the long blocks start first); every warp of a persistent grid takes
- * `chunk` entries at a time from a device counter.  Each block is computed by
- * one warp with the same arithmetic as fsr_reconstruct, so results do not
- * depend on the schedule and equal the single-image results bit for bit. */
+ * `chunk` or more entries at a time from a device counter (more while much of
+ * the list is left).  A list of few blocks (up to 11 per SM) runs as one CTA per
+ * block.  Each block is computed with the same arithmetic as in
+ * fsr_reconstruct, so results do not depend on the schedule and equal the
+ * single-image results bit for bit. */
 
 /* One image of a batch.  Pointer and geometry rules as in fsr_reconstruct. */
 typedef struct fsr_image_desc {
@@ -209,7 +215,7 @@ typedef struct fsr_image_desc {
 /* Schedule of the persistent batch launch. */
 typedef struct fsr_schedule {
     int warps;   /* warps per CTA = support blocks in flight per CTA (FP32: 8, or 12/16 for B = 4; FP64: 4) */
-    int chunk;   /* blocks a warp takes per counter increment, 1..64 */
+    int chunk;   /* least number of blocks a warp takes per counter increment, 1..64 */
 } fsr_schedule;
 
 typedef struct fsr_batch fsr_batch;
@@ -219,9 +225,9 @@ typedef struct fsr_batch fsr_batch;
  * p->seq_out are ignored (per image in d).  The work table lives in
  * handle-owned device memory: a call waits on the host until the previous
  * fsr_reconstruct_batch of this handle has finished before reusing it.
- * With p->reuse > 0 the images run in the re-use form instead: one launch per
- * wavefront index t holds wavefront t of every image that has one (up to 48
- * images per launch), no work table; each image's output equals its
+ * With p->reuse > 0 the images run in the re-use form instead (fsr_params.reuse):
+ * one launch for all, or one launch per wavefront index t that holds wavefront
+ * t of every image that has one (up to 48 images per launch), no work table; each image's output equals its
  * single-image fsr_reconstruct bit for bit.
  * Errors: as fsr_reconstruct, for every image; OOM for the table. */
 int fsr_reconstruct_batch(fsr_handle *h, int n, const fsr_image_desc *d, const fsr_params *p, void *stream);
