@@ -1237,6 +1237,10 @@ __device__ __forceinline__ int image_of(const BatchArgs& a, long long item) {
     return lo;
 }
 
+// A warp's take is 1 / kTakeShare of its equal share of what is left: larger
+// takes leave warps idle at the end, smaller ones cost counter and scan latency
+// (16, 8, 4, 2: 4K, one macroblock in ten lost, K = 50 1.44, 1.39, 1.41, 1.45 ms;
+// 1080p quarter sampling, K = 100 4.59, 4.58, 4.58, 4.97 ms).
 constexpr int kTakeShare = 8;
 
 // Entries a warp takes at once: a share of what is left (so that the warps
