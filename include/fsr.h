@@ -168,9 +168,12 @@ int fsr_reconstruct_host(fsr_handle *h, const float *img, const uint8_t *mask,
  *
  * fsr_check_status synchronises `stream`, then reads and clears the status
  * word: FSR_OK, or FSR_ERR_TIMEOUT with a message when a wait gave up in any
- * single-image launch on h since the last check (a tile copy's, or in the re-use
- * form that of a block row for the row above it, bounded in the same way).  fsr_reconstruct_host does
- * this check itself.  Errors: INVALID_ARG (h NULL), CUDA. */
+ * launch of fsr_reconstruct or fsr_reconstruct_batch on h since the last check:
+ * a tile copy's, or in the re-use form in one launch (fsr_params.reuse) that of a
+ * block row for the row above it.  The latter gives up when no block of the
+ * launch has finished for two seconds (and 4 us per iteration); the rows that
+ * were waiting are left unwritten.  fsr_reconstruct_host does this check itself.
+ * Errors: INVALID_ARG (h NULL), CUDA. */
 int fsr_check_status(fsr_handle *h, void *stream);
 
 /* Test hook (no counterpart in the paper): the next single-image launch on h
@@ -180,6 +183,14 @@ int fsr_check_status(fsr_handle *h, void *stream);
  * the barrier's phase does not.  Launches after it are unaffected.
  * Errors: INVALID_ARG (h NULL). */
 int fsr_inject_tile_wait_fault(fsr_handle *h);
+
+/* Test hook (no counterpart in the paper): the next re-use call on h that runs
+ * in one launch waits with base_ns (0: two seconds) as its base limit; with
+ * skip_first_row nobody takes its first block row, so the rows below it wait in
+ * vain, give up, and the launch ends with FSR_ERR_TIMEOUT from fsr_check_status
+ * (no GPU fault).  Launches after it are unaffected.
+ * Errors: INVALID_ARG (h NULL, base_ns < 0). */
+int fsr_inject_row_wait_fault(fsr_handle *h, long long base_ns, int skip_first_row);
 
 /* Blocks without any known pixel in their support (W[0][0] = 0: no
  * iterations, g = 0, unknown target pixels written as 0; Sec. II, Eq. 10).
@@ -228,7 +239,8 @@ typedef struct fsr_batch fsr_batch;
  * With p->reuse > 0 the images run in the re-use form instead (fsr_params.reuse):
  * one launch for all, or one launch per wavefront index t that holds wavefront
  * t of every image that has one (up to 48 images per launch), no work table; each image's output equals its
- * single-image fsr_reconstruct bit for bit.
+ * single-image fsr_reconstruct bit for bit.  A bounded wait that gave up is
+ * reported by fsr_check_status.
  * Errors: as fsr_reconstruct, for every image; OOM for the table. */
 int fsr_reconstruct_batch(fsr_handle *h, int n, const fsr_image_desc *d, const fsr_params *p, void *stream);
 

@@ -288,7 +288,9 @@ int enqueue_reuse_rows(fsr_handle* h, int n, const fsrk::ImageArgs* ims, const f
     cudaError_t e = h->row_used[slot] ? cudaStreamWaitEvent(stream, h->row_ev[slot], 0) : cudaSuccess;
     if (e == cudaSuccess)
         e = fsrk::launch_coop_rows(method_args(p), p->reuse, n, ims, ring, h->d_status, h->d_empty, p->block,
-                                   h->sm_count, stream);
+                                   h->sm_count, {h->inject_row_base_ns, h->inject_row_skip}, stream);
+    h->inject_row_base_ns = 0;
+    h->inject_row_skip = 0;
     const cudaError_t er = cudaEventRecord(h->row_ev[slot], stream);
     if (er == cudaSuccess) h->row_used[slot] = true;
     if (e == cudaSuccess) e = er;
@@ -777,6 +779,14 @@ int fsr_empty_blocks(fsr_handle* h, void* stream, long long* count) {
 int fsr_inject_tile_wait_fault(fsr_handle* h) {
     if (!h) return fail(nullptr, FSR_ERR_INVALID_ARG, "handle is NULL");
     h->inject_tile_fault = 1;
+    return ok(h);
+}
+
+int fsr_inject_row_wait_fault(fsr_handle* h, long long base_ns, int skip_first_row) {
+    if (!h) return fail(nullptr, FSR_ERR_INVALID_ARG, "handle is NULL");
+    if (base_ns < 0) return fail(h, FSR_ERR_INVALID_ARG, "base_ns is negative");
+    h->inject_row_base_ns = (unsigned long long)base_ns;
+    h->inject_row_skip = skip_first_row != 0;
     return ok(h);
 }
 

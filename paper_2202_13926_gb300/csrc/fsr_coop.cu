@@ -79,10 +79,17 @@ cudaError_t launch_coop(const BatchArgs& a, int B, const ImageArgs* one, int sm_
     }
 }
 
-size_t coop_rows_bytes() { return sizeof(unsigned long long) * (coop::kRowRing + 1); }
+size_t coop_rows_bytes() { return sizeof(unsigned long long) * (coop::kRowRing + 2); }
+
+// A block with `iters` iterations takes up to 0.5 us for each beside three others
+// on its SM (0.2 us alone): eight times that, and two seconds.
+unsigned long long row_limit_ns(unsigned long long base_ns, int iters) {
+    return (base_ns ? base_ns : 2000000000ull) + 4000ull * (unsigned long long)(iters + 16);
+}
 
 cudaError_t launch_coop_rows(const MethodArgs& mth, float delta, int n, const ImageArgs* ims, void* ring,
-                             unsigned* status, unsigned long long* empty, int B, int sm_count, cudaStream_t stream) {
+                             unsigned* status, unsigned long long* empty, int B, int sm_count, RowWaitHook hook,
+                             cudaStream_t stream) {
     coop::RowsArgs a = {};
     a.mth = mth;
     a.delta = delta;
@@ -91,16 +98,20 @@ cudaError_t launch_coop_rows(const MethodArgs& mth, float delta, int n, const Im
     a.status = status;
     a.empty = empty;
     a.n = n;
-    int order[coop::kRowImages];
+    int order[coop::kRowImages], iters = 0;
     for (int i = 0; i < n; ++i) order[i] = i;
     std::stable_sort(order, order + n, [&](int x, int y) { return ims[x].H > ims[y].H; });
     for (int i = 0; i < n; ++i) {
         a.im[i] = ims[order[i]];
         a.nby[i] = (a.im[i].H + B - 1) / B;
         a.rows += a.nby[i];
+        iters = std::max(iters, a.im[i].K);
     }
+    a.limit_ns = row_limit_ns(hook.base_ns, iters);
     const int wanted = (int)coop_rows_parallel(n, ims, mth.L, B);
     cudaError_t e = cudaMemsetAsync(ring, 0, coop_rows_bytes(), stream);
+    if (e == cudaSuccess && hook.skip_row)   // the row counter starts at 1: nobody takes row 0
+        e = cudaMemsetAsync(a.ring + coop::kRowRing, 1, 1, stream);
     if (e != cudaSuccess) return e;
     switch (B) {
         case 2: return launch_rows_b<2>(a, wanted, sm_count, stream);

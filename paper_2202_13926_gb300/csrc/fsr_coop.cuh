@@ -637,7 +637,8 @@ struct RowsArgs {
     MethodArgs mth;
     float delta;
     int lag, n, rows;            // rows of all images together
-    unsigned long long* ring;    // kRowRing entries, then the row counter: zero at launch
+    unsigned long long* ring;    // kRowRing entries, then the row counter and the finished blocks: zero at launch
+    unsigned long long limit_ns; // of the waits
     unsigned* status;
     unsigned long long* empty;
     ImageArgs im[kRowImages];    // by falling number of block rows
@@ -655,10 +656,14 @@ __device__ __forceinline__ void st_release(unsigned long long* p, unsigned long 
 }
 
 // One thread: wait (bounded) until slot shows row g with at least `need`
-// blocks done, or a later row.  The limit is two seconds plus far more than
-// the rows ahead can take (1 us per iteration and block).
-__device__ __forceinline__ bool row_wait(const unsigned long long* slot, unsigned g, unsigned need,
-                                         unsigned long long limit_ns) {
+// blocks done, or a later row.  The wait gives up when no block of the launch
+// has finished for limit_ns (row_limit_ns: more than any block takes).  The
+// row waited for may itself stand still for much longer, behind all rows
+// between it and the one at work, and those may be of an image with other
+// sizes and iterations than this one's: 300 rows of two blocks each, K = 100,
+// start 13 ms after one another's first.
+__device__ __forceinline__ bool row_wait(const RowsArgs& a, unsigned g, unsigned need) {
+    const unsigned long long* slot = a.ring + g % (unsigned)kRowRing;
     unsigned long long t0 = 0, last = 0;
     for (unsigned it = 0;; ++it) {
         const unsigned long long v = ld_acquire(slot);
@@ -666,11 +671,12 @@ __device__ __forceinline__ bool row_wait(const unsigned long long* slot, unsigne
         if (tag > g + 1u || (tag == g + 1u && (unsigned)v >= need)) return true;
         __nanosleep(64);
         if ((it & 63u) == 0u) {
+            const unsigned long long done = ld_acquire(a.ring + kRowRing + 1);
             unsigned long long t;
             asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-            if (it == 0u || v != last) t0 = t;   // the clock starts again whenever the row moves on
-            else if (t - t0 > limit_ns) return false;
-            last = v;
+            if (it == 0u || done != last) t0 = t;   // the clock starts again with every block that finishes
+            else if (t - t0 > a.limit_ns) return false;
+            last = done;
         }
     }
 }
@@ -702,18 +708,16 @@ __global__ void __launch_bounds__(Cfg<4>::T) fsr_coop_rows_kernel(const __grid_c
         const int prev = r > 0 ? before(r - 1) + i : 0;   // row r - 1 of this image
         const ImageArgs im = a.im[i];
         unsigned long long* slot = a.ring + g % kRowRing;
-        const unsigned long long limit =
-            2000000000ull + 1000ull * (unsigned long long)(im.K + 16) * (unsigned long long)(im.nbx + a.lag);
         const unsigned long long tag = (unsigned long long)(g + 1) << 32;
         if (threadIdx.x == 0) {
-            s_ok = g < kRowRing || row_wait(slot, (unsigned)(g - kRowRing), 0xffffffffu, limit);
+            s_ok = g < kRowRing || row_wait(a, (unsigned)(g - kRowRing), 0xffffffffu);
             if (s_ok) st_release(slot, tag);
         }
         __syncthreads();
         for (int bx = 0; bx < im.nbx; ++bx) {
             // the row above, while thread 0 publishes the last block
             if (threadIdx.x == Cfg<4>::T - 1 && r > 0 && s_ok &&
-                !row_wait(a.ring + prev % kRowRing, (unsigned)prev, (unsigned)min(bx + a.lag, im.nbx), limit))
+                !row_wait(a, (unsigned)prev, (unsigned)min(bx + a.lag, im.nbx)))
                 s_ok = 0;
             __syncthreads();
             if (!s_ok) {
@@ -723,7 +727,10 @@ __global__ void __launch_bounds__(Cfg<4>::T) fsr_coop_rows_kernel(const __grid_c
             block<B, 4, true, false>(im, r, bx, a.mth, sm, a.empty, a.delta);
             __syncthreads();
             // (release at the end of a barrier: the CTA's pixels come before it)
-            if (threadIdx.x == 0) st_release(slot, tag | (bx + 1 == im.nbx ? 0xffffffffu : (unsigned)(bx + 1)));
+            if (threadIdx.x == 0) {
+                st_release(slot, tag | (bx + 1 == im.nbx ? 0xffffffffu : (unsigned)(bx + 1)));
+                atomicAdd(a.ring + kRowRing + 1, 1ull);
+            }
         }
     }
 }

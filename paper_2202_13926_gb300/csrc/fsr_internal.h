@@ -78,5 +78,7 @@ struct fsr_handle {
     cudaEvent_t row_ev[kRowSlots] = {};
     bool row_used[kRowSlots] = {};
     unsigned long long row_next = 0;
+    unsigned long long inject_row_base_ns = 0;   // test hook: of the next one-launch re-use call (fsr_inject_row_wait_fault)
+    int inject_row_skip = 0;
     int inject_tile_fault = 0;     // test hook: next tile-copy launch waits for bytes that never come
 };

@@ -81,8 +81,15 @@ cudaError_t launch_coop_reuse(const ReuseLaunch& a, int B, cudaStream_t stream);
 constexpr int kCoopRowsPerSm = 8;
 size_t coop_rows_bytes();
 long long coop_rows_parallel(int n, const ImageArgs* ims, int L, int B);
+// Test hook of the row waits: another base limit (0: the usual one), and
+// a launch whose first row nobody takes.
+struct RowWaitHook {
+    unsigned long long base_ns;
+    int skip_row;
+};
 cudaError_t launch_coop_rows(const MethodArgs& mth, float delta, int n, const ImageArgs* ims, void* ring,
-                             unsigned* status, unsigned long long* empty, int B, int sm_count, cudaStream_t stream);
+                             unsigned* status, unsigned long long* empty, int B, int sm_count, RowWaitHook hook,
+                             cudaStream_t stream);
 
 // Short-lived-CTA form of the FP32 batch kernel (kWarpsFp32 warps, any B),
 // for launches with a.one_round set (the serving loop).

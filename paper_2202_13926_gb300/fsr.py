@@ -39,7 +39,8 @@ EXPORTED = ("fsr_create", "fsr_destroy", "fsr_last_error", "fsr_reconstruct",
             "fsr_autotune_batch", "fsr_get_schedule", "fsr_set_schedule",
             "fsr_reconstruct_batch_static", "fsr_server_create", "fsr_server_submit",
             "fsr_server_poll", "fsr_server_stats", "fsr_server_destroy",
-            "fsr_check_status", "fsr_inject_tile_wait_fault", "fsr_empty_blocks")
+            "fsr_check_status", "fsr_inject_tile_wait_fault", "fsr_inject_row_wait_fault",
+            "fsr_empty_blocks")
 
 
 class FsrError(RuntimeError):
@@ -128,13 +129,14 @@ def load_library(path: str | None = None):
         lib.fsr_server_destroy.argtypes = [vp]
         lib.fsr_check_status.argtypes = [vp, vp]
         lib.fsr_inject_tile_wait_fault.argtypes = [vp]
+        lib.fsr_inject_row_wait_fault.argtypes = [vp, ctypes.c_longlong, ip]
         lib.fsr_empty_blocks.argtypes = [vp, vp, llp]
         for name in ("fsr_server_create", "fsr_server_submit", "fsr_server_poll",
                      "fsr_server_stats", "fsr_server_destroy"):
             getattr(lib, name).restype = ip
         for name in ("fsr_reconstruct_batch_static", "fsr_reconstruct_batch", "fsr_batch_create", "fsr_batch_launch",
                      "fsr_batch_destroy", "fsr_autotune_batch", "fsr_get_schedule",
-                     "fsr_set_schedule", "fsr_check_status", "fsr_inject_tile_wait_fault",
+                     "fsr_set_schedule", "fsr_check_status", "fsr_inject_tile_wait_fault", "fsr_inject_row_wait_fault",
                      "fsr_empty_blocks"):
             getattr(lib, name).restype = ip
         if path is None:
@@ -255,7 +257,8 @@ def _stream_ptr(stream, device=None):
 
 def fsr_check_status(handle, stream=None) -> None:
     """Synchronise ``stream`` and raise FsrError(FSR_ERR_TIMEOUT) when a
-    bounded tile-copy wait of a single-image launch gave up."""
+    bounded wait of a launch gave up (for a tile copy, or of a block row of the
+    re-use form for the row above)."""
     _check(load_library().fsr_check_status(handle, _stream_ptr(stream)), handle)
 
 
@@ -271,6 +274,13 @@ def fsr_inject_tile_wait_fault(handle) -> None:
     """Test hook: the next tile-copy launch on ``handle`` waits for bytes
     that never arrive, so its bounded waits run out (no GPU fault)."""
     _check(load_library().fsr_inject_tile_wait_fault(handle), handle)
+
+
+def fsr_inject_row_wait_fault(handle, base_ns: int = 0, skip_first_row: bool = False) -> None:
+    """Test hook: the next re-use call on ``handle`` that runs in one launch
+    waits with ``base_ns`` as its base limit; with ``skip_first_row`` nobody
+    takes its first block row, so the waits for it run out (no GPU fault)."""
+    _check(load_library().fsr_inject_row_wait_fault(handle, int(base_ns), int(skip_first_row)), handle)
 
 
 def image_desc(img, mask, out, iters: int, seq_out=None) -> fsr_image_desc:
