@@ -147,11 +147,32 @@ __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, 
 __device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
+// (binary64: left to the compiler, no two kernels share results)
+__device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ double add_rn(double a, double b) { return a + b; }
+__device__ __forceinline__ float sub_rn(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ double sub_rn(double a, double b) { return a - b; }
 
 // obj = w_f (Re^2 + Im^2) (Eq. 8 / the objective of Sec. III-B).
 template <typename T>
 __device__ __forceinline__ T objective(T re, T im, T wf) {
     return mul_rn(wf, fma_rn(im, im, mul_rn(re, re)));
+}
+
+// x = b (c + j s) with the twiddle e^{-j 2 pi tw / 32} = c + j s.  In binary32
+// every rounding is written out: the CTA-per-block kernel (fsr_coop.cuh) gives
+// the same bits as the one-warp kernel, so which product of b_r c - b_i s and b_r
+// s + b_i c is fused with the sum must not be the compiler's choice.  b_r c and
+// b_i c are the fused ones, but for tw = 12 b_i s in x_r and for tw = 4 b_r s in
+// x_i: the choice that every result of this library has been computed with.
+__device__ __forceinline__ void twiddle(float br, float bi, float c, float s, int tw, float& xr, float& xi) {
+    const bool t4 = tw == 4, t12 = tw == 12;
+    xr = __fmaf_rn(t12 ? -bi : br, t12 ? s : c, t12 ? __fmul_rn(br, c) : -__fmul_rn(bi, s));
+    xi = __fmaf_rn(t4 ? br : bi, t4 ? s : c, t4 ? __fmul_rn(bi, c) : __fmul_rn(br, s));
+}
+__device__ __forceinline__ void twiddle(double br, double bi, double c, double s, int, double& xr, double& xi) {
+    xr = br * c - bi * s;
+    xi = br * s + bi * c;
 }
 
 // In-register radix-2 decimation-in-time FFT of length 32, natural order in
@@ -180,13 +201,12 @@ __device__ __forceinline__ void fft32(T (&re)[32], T (&im)[32]) {
                     xr = bi; xi = -br;
                 } else {
                     const T c = T(cos_2pi32(tw)), s = T(-sin_2pi32(tw));
-                    xr = br * c - bi * s;
-                    xi = br * s + bi * c;
+                    twiddle(br, bi, c, s, tw, xr, xi);
                 }
-                ar[j + t + half] = ar[j + t] - xr;
-                ai[j + t + half] = ai[j + t] - xi;
-                ar[j + t] = ar[j + t] + xr;
-                ai[j + t] = ai[j + t] + xi;
+                ar[j + t + half] = sub_rn(ar[j + t], xr);
+                ai[j + t + half] = sub_rn(ai[j + t], xi);
+                ar[j + t] = add_rn(ar[j + t], xr);
+                ai[j + t] = add_rn(ai[j + t], xi);
             }
         }
     }
@@ -433,7 +453,7 @@ __device__ __forceinline__ bool transform_block(const ImageArgs& a, int y0, int 
     auto weight = [&](int m) -> T {
         if constexpr (REUSE)
             return ((known >> m) & 1u) ? sw0[m * S + lane]
-                                       : (((reused >> m) & 1u) ? T(ru->delta) * sw0[m * S + lane] : T(0));
+                                       : (((reused >> m) & 1u) ? mul_rn(T(ru->delta), sw0[m * S + lane]) : T(0));
         else
             return ((known >> m) & 1u) ? sw0[m * S + lane] : T(0);
     };
@@ -443,8 +463,8 @@ __device__ __forceinline__ bool transform_block(const ImageArgs& a, int y0, int 
 #pragma unroll
     for (int m = 0; m < S; ++m) {
         const T w = weight(m);
-        sw += w;
-        sfw += w * zr[m];
+        sw = add_rn(sw, w);
+        sfw = fma_rn(w, zr[m], sfw);
         if constexpr (DFT != Dft::SIMT) swd += double(w);
     }
     if (__ballot_sync(FULL, avail != 0) == 0) return false;
@@ -465,8 +485,8 @@ __device__ __forceinline__ bool transform_block(const ImageArgs& a, int y0, int 
     for (int m = 0; m < S; ++m) {
         const bool kn = (avail >> m) & 1u;
         const T w = weight(m);
-        const T d = zr[m] - mu;
-        zr[m] = kn ? d * w : T(0);
+        const T d = sub_rn(zr[m], mu);
+        zr[m] = kn ? mul_rn(d, w) : T(0);
         zi[m] = w;
         const unsigned ab = __float_as_uint((float)d) & 0x7fffffffu;
         dmax = (kn && ab > dmax) ? ab : dmax;
@@ -477,7 +497,7 @@ __device__ __forceinline__ bool transform_block(const ImageArgs& a, int y0, int 
     const T alpha = T(__uint_as_float(aexp << 23));
     const T inv2alpha = T(__uint_as_float((253u - aexp) << 23));   // 1 / (2 alpha)
 #pragma unroll
-    for (int m = 0; m < S; ++m) zi[m] = zi[m] * alpha;
+    for (int m = 0; m < S; ++m) zi[m] = mul_rn(zi[m], alpha);
 
     if constexpr (DFT != Dft::SIMT) {
         // a3 on tensor cores (precision study); lane k ends with Z[k][0..31]
@@ -875,8 +895,8 @@ __device__ __forceinline__ void record_pick(const Pick& pk, float cg, int nu, in
                                             const int (&pm)[TargetPix<B>::P], const int (&pn)[TargetPix<B>::P],
                                             float (&gacc)[TargetPix<B>::P], const PickList* pl, float& cr,
                                             float& ci, bool pair = false) {
-    cr = pk.Rr * cg;
-    ci = pk.Ri * cg;
+    cr = mul_rn(pk.Rr, cg);
+    ci = mul_rn(pk.Ri, cg);
     if (seq != nullptr && lane == 0) seq[nu] = (int16_t)(pk.u * S + pk.v);
     if constexpr (DENSE) {
         if (lane == 0) {
@@ -1067,7 +1087,7 @@ __device__ __forceinline__ T wf_value(const MethodArgs& mth, int k, int l) {
     const T half = T(S) / T(2);
     const T kt = half - fabs(T(k) - half), lt = half - fabs(T(l) - half);
     const T r = sqrt(kt * kt / T(S * S) + lt * lt / T(S * S));
-    const T b = T(1) - sqrt(T(2)) * r;
+    const T b = fma_rn(-sqrt(T(2)), r, T(1));   // written out: see twiddle()
     return b * b;
 }
 

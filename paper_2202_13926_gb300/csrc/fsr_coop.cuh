@@ -126,16 +126,11 @@ __device__ __forceinline__ void tables(const MethodArgs& mth, Smem<N>* sm) {
     if (tid < S) sm->cs[tid] = make_float2(float(cos_2pi32(tid)), float(sin_2pi32(tid)));
 }
 
-// One butterfly of the FFT, twiddle e^{-j 2 pi tw / 32} = c + j s, with the
-// products rounded as in fft32: of each of x_r = b_r c - b_i s and x_i = b_r s
-// + b_i c one product is rounded and the other fused.  fft32's choice is the
-// compiler's: b_r c and b_i c are the fused ones, but for tw = 4 b_r s in x_i
-// and for tw = 12 b_i s in x_r (found by comparing all choices bit for bit).
-// c = 1, s = -0 and c = 0, s = -1 give fft32's multiplication-free cases.
+// One butterfly of the FFT, twiddle e^{-j 2 pi tw / 32} = c + j s, rounded as in
+// fft32.  c = 1, s = -0 and c = 0, s = -1 give its multiplication-free cases.
 __device__ __forceinline__ void butterfly(float2& a, float2& b, float c, float s, int tw) {
-    const bool t4 = tw == 4, t12 = tw == 12;
-    const float xr = __fmaf_rn(t12 ? -b.y : b.x, t12 ? s : c, t12 ? __fmul_rn(b.x, c) : -__fmul_rn(b.y, s));
-    const float xi = __fmaf_rn(t4 ? b.x : b.y, t4 ? s : c, t4 ? __fmul_rn(b.y, c) : __fmul_rn(b.x, s));
+    float xr, xi;
+    twiddle(b.x, b.y, c, s, tw, xr, xi);
     b.x = __fsub_rn(a.x, xr);
     b.y = __fsub_rn(a.y, xi);
     a.x = __fadd_rn(a.x, xr);
