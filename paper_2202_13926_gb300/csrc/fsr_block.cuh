@@ -1271,43 +1271,94 @@ __device__ __forceinline__ int guided_take(const BatchArgs& a, long long seen, i
     return max(least, (int)min(share, 32u));
 }
 
-// Entries base .. base + count - 1 (count <= 32), one per lane: a block whose
-// target pixels are all known is its input copied, whatever the model (end of
-// Sec. II), so its lane copies it here and the block is done (4K, one 16 x 16
-// macroblock in ten lost, S = 32, K = 50: 10.39 -> 1.42 ms).  Returns the
-// entries that need the iteration: those with an unknown target pixel, and
-// those whose selected indices are asked for.
+// Entries base .. base + count - 1 (count <= 32): a block whose target pixels
+// are all known is its input copied, whatever the model (end of Sec. II), so it
+// is copied here and done (4K, one 16 x 16 macroblock in ten lost, S = 32, K = 50:
+// 10.39 -> 1.42 ms).  Returns the entries that need the iteration: those with an
+// unknown target pixel, and those whose selected indices are asked for.
+//
+// A lane per entry reads its rows until one has an unknown pixel: one entry or
+// 32 cost the same.  At B = 16, whose warps take one or two entries at a time,
+// that was a chain of up to 16 loads (1080p, K = 25, 2 % of the pixels lost: 126 us
+// without looking, 147 with it); there the whole warp looks at each entry, all
+// its loads in flight together (125 us; one macroblock in ten lost 76 -> 56 us,
+// half of the pixels lost 126 us all three ways).  At B = 8 that form gained
+// where little is lost (K = 25: 397 -> 357 us) but cost 0.3 to 0.8 % where half is.
 template <int B>
 __device__ __forceinline__ unsigned scan_targets(const BatchArgs& a, long long base, int count, int lane) {
-    const long long item = base + lane;
-    bool need = false;
-    if (lane < count && item < a.total) {
-        const int lo = image_of(a, item);
-        const ImageArgs* im = a.images + lo;
-        const int blk_x = im->nbx, W = im->W, H = im->H, pitch = im->pitch;
-        const long long blk = item - __ldg(a.first + lo);
-        const int by = (int)(blk / blk_x), bx = (int)(blk - (long long)by * blk_x);
-        const int rows = min(B, H - by * B), cols = min(B, W - bx * B);
-        const size_t off = (size_t)by * B * pitch + (size_t)bx * B;
-        const uint8_t* mask = im->mask + off;
-        need = im->seq != nullptr;
-        for (int r = 0; r < rows && !need; ++r) {
-            unsigned known = 1;
+    if constexpr (B == 16) {
+        constexpr int PT = B * B / 32;   // target pixels per lane, consecutive lanes on consecutive pixels
+        unsigned todo = 0;
+        for (int e = 0; e < count; ++e) {
+            const long long item = base + e;
+            const float* img = nullptr;
+            float* out = nullptr;
+            int rows = 0, cols = 0, pitch = 0;
+            bool need = false;
+            if (item < a.total) {
+                const int lo = image_of(a, item);
+                const ImageArgs* im = a.images + lo;
+                const int blk_x = im->nbx;
+                const long long blk = item - __ldg(a.first + lo);
+                const int by = (int)(blk / blk_x), bx = (int)(blk - (long long)by * blk_x);
+                pitch = im->pitch;
+                rows = min(B, im->H - by * B);
+                cols = min(B, im->W - bx * B);
+                const size_t off = (size_t)by * B * pitch + (size_t)bx * B;
+                need = im->seq != nullptr;
+                img = im->img + off;
+                out = im->out + off;
+                const uint8_t* mask = im->mask + off;
+                unsigned known = 1;
 #pragma unroll
-            for (int c = 0; c < B; ++c)
-                if (c < cols) known = __ldg(mask + (size_t)r * pitch + c) != 0 ? known : 0u;
-            need = known == 0;
+                for (int q = 0; q < PT; ++q) {
+                    const int r = (lane + 32 * q) / B, c = lane % B;
+                    if (r < rows && c < cols) known = __ldg(mask + (size_t)r * pitch + c) != 0 ? known : 0u;
+                }
+                need |= known == 0;
+            }
+            if (__ballot_sync(FULL, need) != 0u) {
+                todo |= 1u << e;
+            } else {
+#pragma unroll
+                for (int q = 0; q < PT; ++q) {
+                    const int r = (lane + 32 * q) / B, c = lane % B;
+                    if (r < rows && c < cols) out[(size_t)r * pitch + c] = __ldg(img + (size_t)r * pitch + c);
+                }
+            }
         }
-        if (!need) {
-            const float* img = im->img + off;
-            float* out = im->out + off;
-            for (int r = 0; r < rows; ++r)
-#pragma unroll
+        return todo;
+    } else {
+        const long long item = base + lane;
+        bool need = false;
+        if (lane < count && item < a.total) {
+            const int lo = image_of(a, item);
+            const ImageArgs* im = a.images + lo;
+            const int blk_x = im->nbx, W = im->W, H = im->H, pitch = im->pitch;
+            const long long blk = item - __ldg(a.first + lo);
+            const int by = (int)(blk / blk_x), bx = (int)(blk - (long long)by * blk_x);
+            const int rows = min(B, H - by * B), cols = min(B, W - bx * B);
+            const size_t off = (size_t)by * B * pitch + (size_t)bx * B;
+            const uint8_t* mask = im->mask + off;
+            need = im->seq != nullptr;
+            for (int r = 0; r < rows && !need; ++r) {
+                unsigned known = 1;
+    #pragma unroll
                 for (int c = 0; c < B; ++c)
-                    if (c < cols) out[(size_t)r * pitch + c] = __ldg(img + (size_t)r * pitch + c);
+                    if (c < cols) known = __ldg(mask + (size_t)r * pitch + c) != 0 ? known : 0u;
+                need = known == 0;
+            }
+            if (!need) {
+                const float* img = im->img + off;
+                float* out = im->out + off;
+                for (int r = 0; r < rows; ++r)
+    #pragma unroll
+                    for (int c = 0; c < B; ++c)
+                        if (c < cols) out[(size_t)r * pitch + c] = __ldg(img + (size_t)r * pitch + c);
+            }
         }
+        return __ballot_sync(FULL, need);
     }
-    return __ballot_sync(FULL, need);
 }
 
 // Batch form: every warp takes consecutive entries of the block list
