@@ -32,7 +32,10 @@
 // publish, and the target pixels of the previous pick, are computed while the
 // reductions and loads run.  A branch in this chain costs 40 to 60 cycles even
 // when every thread goes the same way, so the loop has none.  Scalar
-// components instead of pairs: 457; 8 and 16 warps per block: 480-600.
+// components instead of pairs: 457; 8 and 16 warps per block: 480-600.  With two
+// warps and 8 CTAs per SM the 128 registers do not hold the DC phase's rows beside
+// the state: 84 bytes are spilled (B = 16: up to 164), over one local load and store
+// per warp and iteration.
 //
 // Transforms (four warps): the radix-2 decimation-in-time FFT of length 32
 // splits over the warps.  Warp q takes the inputs of rows (columns) = brev2(q)
@@ -262,7 +265,8 @@ __device__ __forceinline__ void block(const ImageArgs& im, int by, int bx, const
                 if constexpr (REUSE) {
                     const int pby = y / B;
                     const bool earlier = pby < by || (pby == by && pbx < bx);
-                    // earlier targets were written by earlier launches: read through L2
+                    // earlier targets were written by other CTAs, of earlier launches or
+                    // of this one (their rows' progress acquired): read through L2
                     if (earlier) pv = __ldcg(im.out + off);
                     reused = !known && earlier;
                 }

@@ -55,7 +55,12 @@ cudaError_t launch_batch_small(const BatchArgs& a, int S, int B, int fp64, int c
 // blocks, us per call with four / two warps / one warp, K = 100 (K = 25): 0.4
 // blocks per SM 27 / 27 / 75; 2.2 39 / 43 / 74; 3.8 47 / 45 / 73; 4.4 64 (29) /
 // 58 (25) / 74 (35); 6.7 78 / 70 / 74 (33 / 29 / 35); 8.1 102 / 90 / 102; 10.5
-// 109 / 103 / 110 (48 / 43 / 47); 13.3 110 / 117 / 108.
+// 109 / 103 / 110 (48 / 43 / 47); 13.3 110 / 117 / 108 (B = 4).  The upper line at
+// the other B, one warp / two warps, K = 100 (K = 25): 7.2 blocks per SM B = 2 74 /
+// 70 (35 / 29), B = 8 74 / 71 (35 / 29), B = 16 86 / 80 (37 / 33); 10.0 109 / 92 (42 /
+// 40), 111 / 100 (48 / 43), 122 / 115 (48 / 47); 10.5 110 / 102 (46 / 44), 109 / 103
+// (42 / 43), 122 / 117 (49 / 49).  A lower line for few iterations gains below K = 10
+// only.
 // A wavefront of the re-use form takes four warps per block up to
 // kCoopReusePerSm blocks per SM (K = 50, ms for n 1080p frames together with
 // the line at 0, 4, 6, 8, 10, 16: n = 8 98, 82, 68, 68, 68, 69; n = 16 103, 97,
@@ -72,7 +77,7 @@ cudaError_t launch_coop2(const BatchArgs& a, int B, const ImageArgs* one, cudaSt
 cudaError_t launch_coop_reuse(const ReuseLaunch& a, int B, cudaStream_t stream);
 // Re-use form in one launch (fsr_coop_rows_kernel), for calls with at most
 // kCoopRowsPerSm block rows at work per SM (ms, a launch per wavefront / one
-// launch: one 1080p frame, K = 100 53.5 / 45.3, now 39.6; n of them, K = 50: n =
+// launch: one 1080p frame, K = 100 53.5 / 45.3, now 39.2; n of them, K = 50: n =
 // 8 (5.1 rows per SM) 69.4 / 57.1, 12 (7.7) 88.0 / 78.0, 16 (10.2) 94.3 / 97.4,
 // 24 113 / 142), over `ring`, device memory of coop_rows_bytes() that no other
 // launch uses meanwhile.

@@ -26,7 +26,7 @@
 // memory; R_w and W from Z[k][l] and conj Z[-k][-l] with commutative operations
 // (exactly Hermitian, as in the oracle).
 //
-// Measured (K = 100, B = 4), 4 lanes per block -> this: 1280 x 720 133 -> 94 us,
+// Measured (K = 100, B = 4), 4 lanes per block -> this: 1280 x 720 128 -> 90 us,
 // 480 x 480 72 -> 50 us, 64 x 64 48 -> 43 us, 1080p 250 -> 182 us; 16.1 -> 10.7
 // instructions per block and iteration (129 per warp, of 8 blocks, then; 344, of
 // 32, now).  What bounds it now: the issue slots and the latency of one
@@ -539,7 +539,7 @@ __device__ __forceinline__ void run_blocks(const BatchArgs& a, int nblk, const f
     __syncwarp();
 }
 
-// 12 warps per SM (3 CTAs of 4, 150 registers): 1280 x 720 94 us; 10 warps 103,
+// 12 warps per SM (3 CTAs of 4, 146 registers): 1280 x 720 94 us at the time; 10 warps 103,
 // 14 (2 CTAs of 7, 128 registers) 117.
 constexpr int kWarpsQuad = 4;
 constexpr int kCtasQuad = 3;

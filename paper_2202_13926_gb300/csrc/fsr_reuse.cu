@@ -6,8 +6,8 @@
 // 114 ms.  FP32 calls of few block rows take one launch for all wavefronts
 // (fsr_coop_rows_kernel) unless they are captured: one 1080p frame, K = 100:
 // 104.0 ms with a warp per block, 53.5 with a CTA per block and a launch per
-// wavefront, 45.2 in one launch, 39.6 since its iteration is packed; six
-// 480 x 270 frames 27.6, 14.7, 11.3 and 9.9 ms; all bit-identical.
+// wavefront, 45.2 in one launch, 39.2 since its iteration is packed; six
+// 480 x 270 frames 27.6, 14.7, 11.3 and 9.8 ms; all bit-identical.
 #include "fsr_reuse.cuh"
 
 namespace fsrk {
